@@ -174,6 +174,9 @@ struct pt_ctx {
     bool dbl = false, plain = false;
     bool gfp32 = false;  // explicit interaction lists on the FP32 group kernels
     int max_deg = 0;     // largest number of quadruplets holding one mode (quadruplet-list paths)
+    bool row = false;    // comb sweeps on the one-chain-per-block kernel (pt_row.cu)
+    void *d_Jrow = nullptr;  // its coupling store (null: the context does not take that path)
+    int *d_order = nullptr;  // chain slots, largest N first
     cudaStream_t stream = nullptr;
     pt_alloc_fn alloc = nullptr;
     pt_free_fn free_ = nullptr;
@@ -285,6 +288,12 @@ int watchdog_sync(pt_ctx *c) {
 }
 
 // ---------------------------------------------------------------------------------- kernels
+// Whether a comb context of default shape sweeps on the one-chain-per-block kernel.
+bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
+    if (dbl) return maxN <= 160;
+    return maxN <= 32 && n_chains <= 6 * (int64_t)sms;
+}
+
 GraphParams graph_params(pt_ctx *c) {
     GraphParams p{};
     p.samples = c->d_samples; p.groups = c->d_groups; p.quads = c->d_quads; p.Jd = c->d_Jq;
@@ -366,6 +375,17 @@ int run_sweeps(pt_ctx *c, int seg) {
         p.snap_a = reinterpret_cast<double2 *>(c->d_snap_a); p.snap_E = c->d_snap_E; p.n_snap_max = c->n_snap_max;
         p.a_total = c->a_total; p.n_chains = c->n_chains;
         CK(launch_plain_sweep(p, c->n_chains, c->stream));
+        return PT_OK;
+    }
+    if (c->row) {
+        RowParams p{};
+        p.samples = c->d_samples; p.chain_sample = c->d_chain_sample; p.order = c->d_order; p.J = c->d_Jrow;
+        p.a = c->d_a; p.E = c->d_E; p.label = c->d_label; p.beta = c->d_beta; p.mc_acc = c->d_mc_acc;
+        p.mc_att = c->d_mc_att; p.R = c->R; p.nT = c->nT; p.maxN = c->maxN; p.seed = c->seed;
+        p.cc = c->cfg.cc_factor; p.ctl = c->d_ctl; p.n_sweeps = seg; p.measure_every = c->cfg.measure_every;
+        p.snap_a = c->d_snap_a; p.snap_E = c->d_snap_E; p.n_snap_max = c->n_snap_max; p.a_total = c->a_total;
+        p.n_chains = c->n_chains; p.trace = c->d_trace;
+        CK(launch_row_sweep(c->dbl, p, c->stream));
         return PT_OK;
     }
     CK(cudaMemsetAsync(c->d_ctl, 0, sizeof(unsigned int), c->stream));  // ticket
@@ -676,6 +696,7 @@ int set_shape(pt_ctx *c, int G, int ncw, int spu) {
     const int bps = c->cfg.blocks_per_sm > 0 ? std::min(c->cfg.blocks_per_sm, occ) : occ;
     c->grid = std::max(1, std::min((int)c->groups.size(), sms * bps));
     c->G = G; c->ncw = ncw; c->spu = spu;
+    c->row = false;
     drop_graphs(c);
     return PT_OK;
 }
@@ -985,8 +1006,9 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     const int chains_ps = replicas * n_T;
     int G = cfg.chains_per_block, ncw = 0;
     if (c->gfp32) G = 8;  // the group kernels hold 8 chains per block
+    int sms = 0;
     {
-        int dev = 0, sms = 0;
+        int dev = 0;
         if (G == 0 && (cudaGetDevice(&dev) != cudaSuccess ||
                        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
             sms = 0;
@@ -1002,7 +1024,9 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     std::vector<SampleLayout> lay(S);
     std::vector<int> bo_all, xtlo_all, mode_all, ebo_all;
     std::vector<uint32_t> binfo_all;
-    int64_t jblocks = 0, a_off = 0, q_off = 0, inc_total = 0;
+    if (!c->plain && !c->gfp32 && cfg.chains_per_block == 0 && cfg.consumer_warps == 0)
+        c->row = row_path(c->dbl, c->maxN, (int64_t)S * chains_ps, sms);
+    int64_t jblocks = 0, a_off = 0, q_off = 0, inc_total = 0, row_total = 0;
     int chain0 = 0;
     for (int s = 0; s < S; ++s) {
         lay[s] = make_layout(c->N[s]);
@@ -1011,6 +1035,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         sd.tab_off = (int)bo_all.size(); sd.blk_off = (int)binfo_all.size(); sd.mode_off = (int)mode_all.size();
         sd.J_off = jblocks; sd.a_off = a_off; sd.q_off = q_off; sd.nq = J_offsets[s + 1] - J_offsets[s];
         sd.inc_off = inc_total;
+        sd.row_off = row_total;
         bo_all.insert(bo_all.end(), lay[s].bo.begin(), lay[s].bo.end());
         xtlo_all.insert(xtlo_all.end(), lay[s].xtlo.begin(), lay[s].xtlo.end());
         xtlo_all.push_back(0);
@@ -1023,6 +1048,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         a_off += (int64_t)c->N[s] * chains_ps;
         q_off += sd.nq;
         inc_total += 4 * sd.nq;
+        row_total += (int64_t)c->N[s] * (c->N[s] / 2) * c->N[s];
         chain0 += chains_ps;
     }
     // xtlo needs ST entries per sample at tab_off; pad to keep offsets aligned with bo (ST+1 entries)
@@ -1083,7 +1109,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         }
         CK(cudaMemcpy(c->d_J, hJ.data(), hJ.size(), cudaMemcpyHostToDevice));
     }
-    if (c->plain || c->gfp32 || c->maxN <= 64) {
+    if (c->plain || c->gfp32 || c->row || c->maxN <= 64) {
         std::vector<int4> hq((size_t)std::max<int64_t>(q_off, 1));
         std::vector<double> hJq((size_t)std::max<int64_t>(q_off, 1));
         std::vector<int> hinc_off, hinc((size_t)std::max<int64_t>(inc_total, 1));
@@ -1158,6 +1184,19 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
 
     if (c->gfp32) CK(graph_prepare(c->maxN, c->max_deg));
+    if (c->row) {
+        c->d_Jrow = dev_alloc(c, (size_t)row_total * c->esize);
+        if (!c->d_Jrow) return bail(fail(c, PT_ENOMEM, "device allocation failed (couplings)"));
+        CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
+        CK(launch_row_pack(c->dbl, c->d_samples, S, c->d_quads, c->d_Jq, c->d_Jrow, c->stream));
+        std::vector<int> order(c->n_chains);
+        for (int i = 0; i < c->n_chains; ++i) order[i] = i;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int x, int y) { return c->N[c->chain_sample[x]] > c->N[c->chain_sample[y]]; });
+        RC(dalloc(c, &c->d_order, c->n_chains));
+        CK(cudaMemcpy(c->d_order, order.data(), c->n_chains * sizeof(int), cudaMemcpyHostToDevice));
+        CK(row_prepare(c->dbl, c->maxN));
+    }
     // ---- persistent grid
     if (!c->plain && !c->gfp32) {
         int dev = 0, sms = 0;
@@ -1544,6 +1583,7 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
                                                  : (c->maxN >= 192 ? 1 : c->maxN >= 96 ? 2 : c->maxN >= 48 ? 8 : 32);
     struct Cand { int G, ncw, spu; };
     std::vector<Cand> cands;
+    if (c->d_Jrow) cands.push_back({0, 0, spu0});  // one chain per block
     const int Gs_f[] = {8, 16, 32}, Gs_d[] = {8, 16};
     const int ncws[] = {3, 7, 9, 11, 15};
     for (int G : (c->dbl ? std::vector<int>(Gs_d, Gs_d + 2) : std::vector<int>(Gs_f, Gs_f + 3))) {
@@ -1556,9 +1596,15 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
-    Cand bestc = {c->G, c->ncw, c->spu};
+    Cand bestc = {c->row ? 0 : c->G, c->row ? 0 : c->ncw, c->spu};
+    auto set = [&](const Cand &cd) {
+        if (cd.G > 0) return set_shape(c, cd.G, cd.ncw, cd.spu);
+        c->row = true;
+        drop_graphs(c);
+        return (int)PT_OK;
+    };
     for (const Cand &cd : cands) {
-        if (set_shape(c, cd.G, cd.ncw, cd.spu) != PT_OK) continue;
+        if (set(cd) != PT_OK) continue;
         if ((rc = pt_sweep(c, 1)) != PT_OK) break;  // warm-up (graph capture)
         if (cudaEventRecord(e0, c->stream) != cudaSuccess) break;
         if ((rc = pt_sweep(c, trial_sweeps)) != PT_OK) break;
@@ -1570,7 +1616,7 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    const int rc2 = set_shape(c, bestc.G, bestc.ncw, bestc.spu);
+    const int rc2 = set(bestc);
     const int rc3 = pt_load(c, blob.data(), len);  // the trials leave no trace
     if (rc != PT_OK) return rc;
     if (rc2 != PT_OK) return rc2;

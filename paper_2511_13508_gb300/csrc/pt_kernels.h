@@ -166,6 +166,36 @@ cudaError_t launch_graph_sweep(const GraphParams &p, int n_groups, cudaStream_t 
 cudaError_t launch_graph_energy(const GraphParams &p, int n_groups, cudaStream_t s);
 cudaError_t graph_prepare(int maxN, int max_deg);  // shared-memory limits of the graph kernels (N <= maxN)
 
+// pt_row.cu: one chain per block, pair products resident in shared memory (FP64, and FP32 at small N)
+constexpr int kRowMaxThreads = 352;  // N <= 160: ten row warps and the helper
+struct RowParams {
+    const SampleDev *samples;
+    const int *chain_sample;
+    const int *order;        // block -> chain slot, chains of the largest N first
+    const void *J;           // couplings J_l[p][m] per sample at row_off, [N][N/2][N] (float or double)
+    void *a;
+    double *E;
+    const int *label;
+    const double *beta;
+    unsigned long long *mc_acc, *mc_att;
+    int R, nT, maxN;
+    uint64_t seed;
+    double cc;
+    Control *ctl;
+    int n_sweeps, measure_every;
+    void *snap_a;
+    double *snap_E;
+    int n_snap_max;
+    int64_t a_total;
+    int n_chains;
+    double *trace;           // update trace, as SweepParams::trace
+};
+size_t row_smem_bytes(bool dbl, int maxN);
+cudaError_t row_prepare(bool dbl, int maxN);
+cudaError_t launch_row_pack(bool dbl, const SampleDev *samples, int S, const int4 *quads, const double *Jq, void *out,
+                            cudaStream_t s);
+cudaError_t launch_row_sweep(bool dbl, const RowParams &p, cudaStream_t s);
+
 struct PlainParams {
     const SampleDev *samples;
     const int *chain_sample;
