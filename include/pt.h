@@ -215,17 +215,21 @@ int pt_load(pt_ctx *ctx, const void *buf, size_t len);
 /* Autotuner of the sweep blocks (chains per block, field warps, sweeps per scheduling unit): times
  * every supported shape for trial_sweeps sweeps on the live ensemble, keeps the fastest and restores
  * the ensemble (state, counters, accumulators) exactly as before the call.  chosen (optional, 3 ints)
- * receives {chains_per_block, consumer_warps, sweeps_per_unit}.  PT_EUNSUPPORTED for the plain path. */
+ * receives {chains_per_block, consumer_warps, sweeps_per_unit}, {0, 0, sweeps_per_unit} when one chain per block (which
+ * pt_create takes by itself for those ensembles) is the fastest.  PT_EUNSUPPORTED for the plain path. */
 int pt_autotune(pt_ctx *ctx, int trial_sweeps, int *chosen);
 
-/* The sweep-block shape pt_create picks when pt_config.chains_per_block and consumer_warps are 0, for a batch of
- * n_samples samples whose largest mode count is max_n (even, 4..512), chains_per_sample = replicas x
- * temperatures, on a device with sm_count multiprocessors (0: unknown).  Host-only, no device call: writes
- * *chains_per_block (8, 16 or 32) and *consumer_warps.  The rule (measured on GB300): 8 chains from N = 160 on;
- * for 48 <= N < 160 the most chains per block (32 below N = 96, else 16, then 8) that still give at least 0.8 x
- * sm_count groups; 16 chains below N = 48; 8 when a sample has at most 8 chains; 11 field warps from N = 48 on,
- * else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL
- * otherwise, and for out-of-range arguments or NULL outputs). */
+/* The sweep-block shape of a batch by size alone: of n_samples samples whose largest mode count is max_n (even,
+ * 4..512), chains_per_sample = replicas x temperatures, on a device with sm_count multiprocessors (0: unknown).
+ * Host-only, no device call: writes *chains_per_block (8, 16 or 32) and *consumer_warps.  The rule (measured on GB300):
+ * 8 chains from N = 160 on; for 48 <= N < 160 the most chains per block (32 below N = 96, else 16, then 8) that still
+ * give at least 0.8 x sm_count groups; 16 chains below N = 48; 8 when a sample has at most 8 chains; 11 field warps from
+ * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block and consumer_warps 0, pt_create
+ * starts from it and departs where another kernel or shape measured faster: FP64 up to N = 160 and small FP32
+ * ensembles up to N = 48 sweep one chain per block; FP32 ensembles of at most sm_count groups of 8 chains take 8 chains
+ * per block, on clusters of blocks where an update has work for several; and below N = 48 it takes the most chains per
+ * block that fill the device.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL otherwise, and for out-of-range
+ * arguments or NULL outputs). */
 int pt_default_shape(int precision, int max_n, int n_samples, int chains_per_sample, int sm_count,
                      int *chains_per_block, int *consumer_warps);
 

@@ -177,6 +177,7 @@ struct pt_ctx {
     bool row = false;    // comb sweeps on the one-chain-per-block kernel (pt_row.cu)
     void *d_Jrow = nullptr;  // its coupling store (null: the context does not take that path)
     int *d_order = nullptr;  // chain slots, largest N first
+    int cl = 1;              // thread blocks per group (FP32 comb sweep)
     cudaStream_t stream = nullptr;
     pt_alloc_fn alloc = nullptr;
     pt_free_fn free_ = nullptr;
@@ -289,9 +290,25 @@ int watchdog_sync(pt_ctx *c) {
 
 // ---------------------------------------------------------------------------------- kernels
 // Whether a comb context of default shape sweeps on the one-chain-per-block kernel.
+// FP64: wherever its pair products fit in shared memory.  It was the faster one at every size measured on GB300 (us per
+// sweep against 16 x 3 / 8 x 7 blocks): N = 16, 64 chains 18.5 | 268 / 309; N = 64, 1024 chains 890 | 4187 / 2230, 4096
+// chains 3460 | 6110 / 8690; N = 128, 512 chains 3010 | 24500 / 10270.
+// FP32: as long as few chains share an SM, since a block then waits on latencies that sharing couplings does not
+// shorten (168 chains, against the best block shape: N = 16 6.0 | 13.4, N = 32 14.0 | 32, N = 48 40 | 56, N = 64 69 | 70;
+// 1024 chains: N = 16 7.9 | 13.2, N = 32 30 | 34, N = 40 51 | 43; 4096 chains: N = 16 27 | 13.7).
 bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
     if (dbl) return maxN <= 160;
-    return maxN <= 32 && n_chains <= 6 * (int64_t)sms;
+    return maxN <= 48 && n_chains <= (maxN <= 32 ? 6 : 2) * (int64_t)sms;
+}
+
+// Blocks per group of the FP32 sweep (a cluster) when its groups leave SMs idle: the most that keep all groups resident
+// at once, and no more than an update has chunks for.  Measured on GB300 (us per sweep of one sample, 8 chains x 7
+// warps, 1 / 2 / 4 / 8 blocks): N = 256, 12 groups 1680 / 1057 / 633 / 428; N = 160, 8 groups 509 / 349 / 247 / 180;
+// N = 128 306 / 217 / 161 / 144; N = 96, 21 groups 170 / 138 / 107 / 161; N = 64, 21 groups 78 / 71 / 70 / 106.
+int cluster_blocks(int G, int ncw, int maxN, int groups, int sms) {
+    for (int cl = maxN >= 128 ? 8 : maxN >= 64 ? 4 : 1; cl > 1; cl /= 2)
+        if (comb_variant_exists(G, ncw, cl) && groups * cl <= sms && groups <= comb_clusters(G, ncw, cl, maxN, sms)) return cl;
+    return 1;
 }
 
 GraphParams graph_params(pt_ctx *c) {
@@ -400,7 +417,8 @@ int run_sweeps(pt_ctx *c, int seg) {
     p.n_snap_max = c->n_snap_max; p.a_total = c->a_total; p.n_chains = c->n_chains; p.trace = c->d_trace;
     const int units = ((seg + p.sweeps_per_unit - 1) / p.sweeps_per_unit) * p.n_groups;
     const int grid = std::max(1, std::min(c->grid, units));
-    CK(launch_sweep(c->dbl, c->G, c->ncw, p, grid, c->stream));
+    if (!c->dbl) CK(launch_comb(c->G, c->ncw, c->cl, p, grid, c->stream));
+    else CK(launch_sweep(c->dbl, c->G, c->ncw, p, grid, c->stream));
     return PT_OK;
 }
 
@@ -682,19 +700,32 @@ void drop_graphs(pt_ctx *c) {
     c->graph_defs.clear();
 }
 
+// Groups of G chains the device sweeps at once on blocks of ncw field warps, cl blocks per group (0: does not fit).
+int shape_groups(pt_ctx *c, int G, int ncw, int cl, int sms) {
+    if (c->dbl) return sms * sweep_occupancy(true, G, ncw, c->maxN);
+    return comb_clusters(G, ncw, cl, c->maxN, sms);
+}
+bool shape_exists(bool dbl, int G, int ncw) {
+    return dbl ? sweep_variant_exists(true, G, ncw) : comb_variant_exists(G, ncw, 1);
+}
+
 // Switches the sweep blocks to G chains x ncw field warps (sweeps_per_unit spu); rebuilds the groups.
 int set_shape(pt_ctx *c, int G, int ncw, int spu) {
-    if (!sweep_variant_exists(c->dbl, G, ncw)) return fail(c, PT_EINVAL, "unsupported sweep block shape");
-    const int occ = sweep_occupancy(c->dbl, G, ncw, c->maxN);
-    if (occ < 1) return fail(c, PT_EUNSUPPORTED, "sweep block shape does not fit on this GPU");
-    make_groups(c, G);
-    if (c->groups.size() > c->max_groups) return fail(c, PT_EINVAL, "too many groups for this context");
-    CK(cudaMemcpy(c->d_groups, c->groups.data(), c->groups.size() * sizeof(GroupDev), cudaMemcpyHostToDevice));
+    if (!shape_exists(c->dbl, G, ncw)) return fail(c, PT_EINVAL, "unsupported sweep block shape");
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int bps = c->cfg.blocks_per_sm > 0 ? std::min(c->cfg.blocks_per_sm, occ) : occ;
-    c->grid = std::max(1, std::min((int)c->groups.size(), sms * bps));
+    make_groups(c, G);
+    if (c->groups.size() > c->max_groups) return fail(c, PT_EINVAL, "too many groups for this context");
+    c->cl = c->dbl || c->cfg.blocks_per_sm > 0 ? 1 : cluster_blocks(G, ncw, c->maxN, (int)c->groups.size(), sms);
+    int most = shape_groups(c, G, ncw, c->cl, sms);
+    if (most < 1) {
+        make_groups(c, c->G);
+        return fail(c, PT_EUNSUPPORTED, "sweep block shape does not fit on this GPU");
+    }
+    CK(cudaMemcpy(c->d_groups, c->groups.data(), c->groups.size() * sizeof(GroupDev), cudaMemcpyHostToDevice));
+    if (c->cfg.blocks_per_sm > 0) most = std::min(most, sms * c->cfg.blocks_per_sm);
+    c->grid = std::max(1, std::min((int)c->groups.size(), most));
     c->G = G; c->ncw = ncw; c->spu = spu;
     c->row = false;
     drop_graphs(c);
@@ -878,6 +909,27 @@ static void default_shape(bool dbl, int maxN, int S, int chains_ps, int sms, int
     else *ncw_out = (maxN >= 48) ? 11 : 7;
 }
 
+// FP32 shape where nothing is asked for: pt_default_shape's rule, except that
+// - an ensemble of no more groups of 8 than SMs gives each of them a block, or a cluster of blocks of 7 warps (a block's
+//   update takes as long for 8 chains as for 32 when it is alone on its SM: N = 64, 168 chains 78 us per sweep with 8
+//   chains a block, 71 on clusters of 4, 162 with 32 chains);
+// - below N = 48 it takes the most chains per block that still fill the SMs (N = 32, 4096 chains: 39.6 us with 32
+//   chains x 7 warps, 64.7 with 16 x 7; N = 16: 13.2, 28.1).
+static void tuned_shape(int maxN, int S, int chains_ps, int sms, int *G, int *ncw) {
+    if (sms < 1) return;
+    const int64_t g8 = (int64_t)S * ((chains_ps + 7) / 8);
+    if (g8 <= sms) {
+        *G = 8;
+        *ncw = maxN < 48 || cluster_blocks(8, 7, maxN, (int)g8, sms) > (maxN >= 160 ? 2 : 1) ? 7 : 11;
+        return;
+    }
+    if (maxN >= 48) return;
+    *G = 8;
+    for (int g : {32, 16})
+        if (*G == 8 && chains_ps > g / 2 && (int64_t)S * ((chains_ps + g - 1) / g) >= (int64_t)sms * 4 / 5) *G = g;
+    *ncw = 7;
+}
+
 int pt_default_shape(int precision, int max_n, int n_samples, int chains_per_sample, int sm_count,
                      int *chains_per_block, int *consumer_warps) {
     if ((precision != PT_PREC_FP32 && precision != PT_PREC_FP64) || max_n < 4 || max_n > 512 || (max_n & 1) ||
@@ -1009,13 +1061,16 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     int sms = 0;
     {
         int dev = 0;
-        if (G == 0 && (cudaGetDevice(&dev) != cudaSuccess ||
-                       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
             sms = 0;
+        }
+        const bool tuned = !c->dbl && !c->gfp32 && G == 0 && cfg.consumer_warps == 0 && cfg.blocks_per_sm == 0;
         default_shape(c->dbl, c->maxN, S, chains_ps, sms, G, &G, &ncw);
+        if (tuned) tuned_shape(c->maxN, S, chains_ps, sms, &G, &ncw);
     }
     if (cfg.consumer_warps > 0) ncw = cfg.consumer_warps;
-    if (!c->plain && !c->gfp32 && !sweep_variant_exists(c->dbl, G, ncw)) return bail(fail(c, PT_EINVAL, "pt_create: unsupported chains_per_block"));
+    if (!c->plain && !c->gfp32 && !shape_exists(c->dbl, G, ncw)) return bail(fail(c, PT_EINVAL, "pt_create: unsupported chains_per_block"));
     c->G = G; c->ncw = ncw;
     c->spu = cfg.sweeps_per_unit > 0 ? cfg.sweeps_per_unit
                                      : (c->maxN >= 192 ? 1 : c->maxN >= 96 ? 2 : c->maxN >= 48 ? 8 : 32);
@@ -1202,10 +1257,11 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         int dev = 0, sms = 0;
         CK(cudaGetDevice(&dev));
         CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int occ = sweep_occupancy(c->dbl, G, ncw, c->maxN);
-        if (occ < 1) return bail(fail(c, PT_EUNSUPPORTED, "pt_create: sweep kernel does not fit on this GPU for this N"));
-        const int bps = cfg.blocks_per_sm > 0 ? std::min(cfg.blocks_per_sm, occ) : occ;
-        c->grid = std::max(1, std::min((int)c->groups.size(), sms * bps));
+        c->cl = c->dbl || cfg.blocks_per_sm > 0 ? 1 : cluster_blocks(G, ncw, c->maxN, (int)c->groups.size(), sms);
+        int most = shape_groups(c, G, ncw, c->cl, sms);
+        if (most < 1) return bail(fail(c, PT_EUNSUPPORTED, "pt_create: sweep kernel does not fit on this GPU for this N"));
+        if (cfg.blocks_per_sm > 0) most = std::min(most, sms * cfg.blocks_per_sm);
+        c->grid = std::max(1, std::min((int)c->groups.size(), most));
         c->sms = sms;
         RC(dalloc(c, &c->d_epart, c->max_groups * (size_t)kEnergyPartsMax * 32));
     }
@@ -1589,7 +1645,7 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
     for (int G : (c->dbl ? std::vector<int>(Gs_d, Gs_d + 2) : std::vector<int>(Gs_f, Gs_f + 3))) {
         if (G > 8 && cps < G / 2) continue;  // mostly empty blocks
         for (int n : ncws)
-            if (sweep_variant_exists(c->dbl, G, n))
+            if (shape_exists(c->dbl, G, n))
                 for (int sp : {spu0, spu0 * 4}) cands.push_back({G, n, sp});
     }
     cudaEvent_t e0, e1;

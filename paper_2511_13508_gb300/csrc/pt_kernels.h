@@ -71,6 +71,11 @@ struct EnergyParams {
 };
 constexpr int kEnergyPartsMax = 8;
 
+// pt_comb.cu: FP32 comb sweep, G chains per group (on a cluster of cl blocks), ncw field warps per block
+bool comb_variant_exists(int G, int ncw, int cl);
+cudaError_t launch_comb(int G, int ncw, int cl, const SweepParams &p, int clusters, cudaStream_t s);
+int comb_clusters(int G, int ncw, int cl, int maxN, int sms);  // clusters the device holds at once (0: does not fit)
+
 // pt_sweep.cu
 bool sweep_variant_exists(bool dbl, int G, int ncw);
 cudaError_t launch_sweep(bool dbl, int G, int ncw, const SweepParams &p, int grid, cudaStream_t s);

@@ -1,4 +1,4 @@
-// pt_sweep.cu -- the J-sharing Metropolis sweep kernel (sm_103a), its field-only twin and the
+// pt_sweep.cu -- the J-sharing FP64 Metropolis sweep kernel (sm_103a), the field-only kernel and the
 // full-energy (resync) kernel, for the smoothed-cubic 4-body random-laser model (arXiv 2511.13508).
 //
 // Local field of the updated modes (paper Sec. III.A.3).  With z_P = a_x a_y for the pair P = {x,y},
@@ -14,64 +14,12 @@
 //     B_jk = sum_s conj(a_{s-j}) J_j[s][{k, s-k}] a_{s-k},   A_jk = acc_j[j+k].
 #include <cstdint>
 #include <cstdio>
+#include "pt_bulk.cuh"
 #include "pt_common.cuh"
 #include "pt_kernels.h"
 #include "pt_move.cuh"
 
 namespace ptgb {
-
-// ------------------------------------------------------------------------------------------------
-// PTX wrappers: mbarrier, bulk copy, named barriers
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
-                     smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: gives up after kWaitNs of wall time, records the error and reports failure.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, Control *ctl, int where,
-                                                  volatile int *abort_flag) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (uint32_t n = 1;; ++n) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-        if ((n & 63u) == 0 && global_ns() - t0 > kWaitNs) {
-            record_error(ctl, kErrTimeout, where);
-            *abort_flag = 1;
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ void bulk_g2s(void *dst_smem, const void *src_gmem, uint32_t bytes, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst_smem)),
-        "l"(src_gmem), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ void named_bar(int id, int nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 // Row-stride of the shared amplitude table [x + APAD][chain] (complex elements): one pad element for
 // 8-byte complex with 8 chains, so that four workers reading rows 8 apart hit distinct bank halves.
@@ -181,153 +129,6 @@ __device__ __forceinline__ void process_block(const typename vec2<real>::type *_
     }
 }
 
-// ------------------------------------------------------------------------------------------------
-// Packed-FP32 block arithmetic (the FP32 shapes of 8 chains per block).  Rows are taken in pairs (r, r+1)
-// and every quantity is a float2 pair over the two rows, so each instruction is an FFMA2/FMUL2 doing two
-// fused multiply-adds: with
-//     sx = (Re a_x, Re a_x), sy = (Im a_x, Im a_x)                  (splats of a_x in registers)
-//     WX = (Re a_y, Re a_{y+1}), WY = (Im a_y, Im a_{y+1})          (window table awin, y = s - x)
-// the pair products of rows (s, s+1) at column x are
-//     Re z = sx WX - sy WY,   Im z = sx WY + sy WX,
-// and a field row pair accumulates acc += (J[s][x], J[s+1][x]) z with the column-major J block supplying
-// the coupling pair directly.  Two FMUL2 + two FFMA2 make 2 products; one FFMA2 per field per component
-// accumulates them: 2 instructions per coupling term when both fields use the block, 3 otherwise.
-struct PartialsX2 {
-    float2 hjx, hjy, hjyn, hkx, hky, hkyn;  // h = (hx.0 + hx.1, (hy.0 + hy.1) - (hyn.0 + hyn.1))
-    float2 B, A;
-    __device__ __forceinline__ void zero() {
-        hjx = hjy = hjyn = hkx = hky = hkyn = B = A = make_float2(0.f, 0.f);
-    }
-};
-
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-
-template <int G, int MODE, bool WB>
-__device__ __forceinline__ void process_block_x2(const float2 *__restrict__ as, const float4 *__restrict__ awin,
-                                                 int c, int s0, int x0, int j, int k, int N, const float *Jj,
-                                                 const float *Jk, PartialsX2 &p) {
-    constexpr int RS = RowStride<float, G>::value;
-    // Column i = 2h + pi pairs rows (2q, 2q+1) with the window starting at y-offset d = 2q - i + 7, of parity
-    // 1 - pi: the columns run in two passes by parity, each holding the 7 windows of its parity
-    // (d = 2m + 1 - pi, m = q - h + 3), so that only 7 windows are live at a time.
-    const int ybase = s0 - x0 - (TX - 1) + APAD;
-    float2 ajx[TS / 2], ajy[TS / 2], akx[TS / 2], aky[TS / 2];
-#pragma unroll
-    for (int q = 0; q < TS / 2; ++q) ajx[q] = ajy[q] = akx[q] = aky[q] = f2(0.f, 0.f);
-#pragma unroll
-    for (int pi = 0; pi < 2; ++pi) {
-        float2 wx[7], wy[7];
-#pragma unroll
-        for (int m = 0; m < 7; ++m) {
-            const float4 w = awin[(ybase + 2 * m + 1 - pi) * G + c];
-            wx[m] = f2(w.x, w.y);
-            wy[m] = f2(w.z, w.w);
-        }
-#pragma unroll
-        for (int h = 0; h < TX / 2; ++h) {
-            const int i = 2 * h + pi;
-            // splats of a_x in registers (register moves cost less than the shared-memory bandwidth of a table)
-            const float2 axv = as[(x0 + i + APAD) * RS + c];
-            const float2 sx = f2(axv.x, axv.x), sy = f2(axv.y, axv.y), nsy = f2(-axv.y, -axv.y);
-            float2 jp[TS / 2], kp[TS / 2];
-            if (MODE & 1) {
-                const float4 a = *reinterpret_cast<const float4 *>(Jj + i * TS), b = *reinterpret_cast<const float4 *>(Jj + i * TS + 4);
-                jp[0] = f2(a.x, a.y); jp[1] = f2(a.z, a.w); jp[2] = f2(b.x, b.y); jp[3] = f2(b.z, b.w);
-            }
-            if (MODE & 2) {
-                const float4 a = *reinterpret_cast<const float4 *>(Jk + i * TS), b = *reinterpret_cast<const float4 *>(Jk + i * TS + 4);
-                kp[0] = f2(a.x, a.y); kp[1] = f2(a.z, a.w); kp[2] = f2(b.x, b.y); kp[3] = f2(b.z, b.w);
-            }
-            float2 tx[TS / 2], ty[TS / 2], zx[TS / 2], zy[TS / 2];
-#pragma unroll
-            for (int q = 0; q < TS / 2; ++q) {
-                const int m = q - h + 3;
-                tx[q] = __fmul2_rn(nsy, wy[m]);
-                ty[q] = __fmul2_rn(sy, wx[m]);
-            }
-#pragma unroll
-            for (int q = 0; q < TS / 2; ++q) {
-                const int m = q - h + 3;
-                zx[q] = __ffma2_rn(sx, wx[m], tx[q]);
-                zy[q] = __ffma2_rn(sx, wy[m], ty[q]);
-            }
-#pragma unroll
-            for (int q = 0; q < TS / 2; ++q) {
-                if (MODE & 1) { ajx[q] = __ffma2_rn(jp[q], zx[q], ajx[q]); ajy[q] = __ffma2_rn(jp[q], zy[q], ajy[q]); }
-                if (MODE & 2) { akx[q] = __ffma2_rn(kp[q], zx[q], akx[q]); aky[q] = __ffma2_rn(kp[q], zy[q], aky[q]); }
-            }
-        }
-    }
-    // close the rows: h += conj(m) acc with m = a_{s-l} for the row pair (s, s+1) from the window table
-#pragma unroll
-    for (int q = 0; q < TS / 2; ++q) {
-        if (MODE & 1) {
-            const float4 w = awin[(s0 + 2 * q - j + APAD) * G + c];
-            const float2 mx = f2(w.x, w.y), my = f2(w.z, w.w);
-            p.hjx = __ffma2_rn(mx, ajx[q], p.hjx);
-            p.hjx = __ffma2_rn(my, ajy[q], p.hjx);
-            p.hjy = __ffma2_rn(mx, ajy[q], p.hjy);
-            p.hjyn = __ffma2_rn(my, ajx[q], p.hjyn);
-        }
-        if (MODE & 2) {
-            const float4 w = awin[(s0 + 2 * q - k + APAD) * G + c];
-            const float2 mx = f2(w.x, w.y), my = f2(w.z, w.w);
-            p.hkx = __ffma2_rn(mx, akx[q], p.hkx);
-            p.hkx = __ffma2_rn(my, aky[q], p.hkx);
-            p.hky = __ffma2_rn(mx, aky[q], p.hky);
-            p.hkyn = __ffma2_rn(my, akx[q], p.hkyn);
-        }
-    }
-    if (MODE & 1) {
-        // A_jk is the accumulator of row j+k
-        const int rs = j + k - s0;
-        if (rs >= 0 && rs < TS) {
-#pragma unroll
-            for (int q = 0; q < TS / 2; ++q) {
-                if (rs == 2 * q) { p.A.x += ajx[q].x; p.A.y += ajy[q].x; }
-                if (rs == 2 * q + 1) { p.A.x += ajx[q].y; p.A.y += ajy[q].y; }
-            }
-        }
-    }
-    if ((MODE & 1) && WB) {
-        const bool col = (k >= x0 && k < x0 + TX);
-        const bool diag = (s0 + TS - 1 >= x0 + k) && (s0 <= x0 + TX - 1 + k);
-        if (col || diag) {
-#pragma unroll
-            for (int r = 0; r < TS; ++r) {
-                const int s = s0 + r, y = s - k;
-                const int xs = (y < k) ? y : k;
-                if (y >= 0 && y < N && xs >= x0 && xs < x0 + TX) {
-                    const float Jv = Jj[(xs - x0) * TS + r];
-                    const float2 m = as[(s - j + APAD) * RS + c];
-                    const float2 yv = as[(y + APAD) * RS + c];
-                    caxpy(p.B, Jv, cmulc(m, yv));
-                }
-            }
-        }
-    }
-}
-
-template <int G, bool WB>
-__device__ __forceinline__ void process_block_x2_dispatch(int mode, const float2 *as, const float4 *awin, int c,
-                                                          int s0, int x0, int j, int k, int N, const float *Jj,
-                                                          const float *Jk, PartialsX2 &p) {
-    if (mode == 3) process_block_x2<G, 3, WB>(as, awin, c, s0, x0, j, k, N, Jj, Jk, p);
-    else if (mode == 1) process_block_x2<G, 1, WB>(as, awin, c, s0, x0, j, k, N, Jj, Jk, p);
-    else if (mode == 2) process_block_x2<G, 2, WB>(as, awin, c, s0, x0, j, k, N, Jj, Jk, p);
-}
-
-// Window entry of one amplitude-table row (shared-memory row index R = x + APAD): (Re a_R, Re a_{R+1},
-// Im a_R, Im a_{R+1}).
-template <int RS>
-__device__ __forceinline__ void packed_rows(const float2 *as, float4 *awin, int G, int R, int rows, int c) {
-    const float2 a = as[R * RS + c];
-    const float2 b = (R + 1 < rows) ? as[(R + 1) * RS + c] : make_float2(0.f, 0.f);
-    awin[R * G + c] = make_float4(a.x, b.x, a.y, b.y);
-}
-
-// WB: also pick the B_jk elements out of the block (the field-only kernel); the sweep kernel gathers them
-// once per update instead (b_couplings).
 template <typename real, int RS, bool WB>
 __device__ __forceinline__ void process_block_dispatch(int mode, const typename vec2<real>::type *as, int c,
                                                        int s0, int x0, int j, int k, int N, const real *Jj,
@@ -356,30 +157,9 @@ __device__ __forceinline__ Ranges update_ranges(const SampleDev &sd, const int *
     return R;
 }
 
-// Smallest N for which the FP32 sweep kernel gathers the B_jk couplings once per update (b_coupling, by the copy
-// warp into a shared buffer) instead of picking them out of the blocks.  Measured on GB300 (chain-sweeps/s): with
-// the gather from N = 48 on every FP32 shape, the ragged batch on 16 x 11 8.72M -> 8.82M and on 8 x 11 8.53M ->
-// 8.62M, the others unchanged; when the field warps still did the gather themselves it paid only from N = 128 on.
-constexpr int kGatherBMinN = 48;
-template <typename real, int G> constexpr bool kGatherB = sizeof(real) == 4;
-// With 8 chains per block the copy warp also draws the random part of every chain's proposal, up to kBD updates
-// ahead, and warp 0 only finishes it at the update's start (measured on GB300: N = 256 bench workload +0.8%;
-// with 16 or 32 chains per block warp 0 drawing the whole proposal itself measured 0.7-1.5% faster).
+// With 8 chains per block the copy warp also draws the random part of every chain's proposal, up to kBD updates ahead,
+// and warp 0 only finishes it at the update's start; with 16 chains warp 0 draws the whole proposal itself.
 template <int G> constexpr bool kCopyDraws = G == 8;
-
-// The coupling J_j[s][{k, s-k}] of quadruplet {j, s-j, k, s-k} (0 where the store holds no such entry):
-// column x* = min(k, s-k) of row s in mode j's run, read from global memory (L2-resident: the run is
-// being streamed for the same update).
-template <typename real>
-__device__ __forceinline__ real b_coupling(const real *__restrict__ J, const int *s_bo, const int *s_xtlo,
-                                           const Ranges &Rg, int s, int k) {
-    const int y = s - k, x = y < k ? y : k;
-    const int st = s / TS, xt = x / TX;
-    const int xi = xt - s_xtlo[st];
-    if (xi < 0 || xi >= s_bo[st + 1] - s_bo[st]) return real(0);
-    const int64_t gb = Rg.jg + (s_bo[st] + xi - Rg.jlo);
-    return __ldg(J + gb * JStride<real>::value + (x - xt * TX) * TS + (s - st * TS));
-}
 
 template <typename real>
 __device__ __forceinline__ real delta_h(const Proposal<real> &P, const Partials<real> &f, real cc) {
@@ -418,18 +198,17 @@ __device__ __noinline__ void trace_write(double *trace, int n_chains, int64_t a_
 }
 
 // ------------------------------------------------------------------------------------------------
-// The persistent sweep kernel.  NCW consumer warps + 1 producer warp.  A consumer lane is
+// The persistent FP64 sweep kernel of explicit block shapes and of N > 160 (the others run one chain per block,
+// pt_row.cu; FP32: pt_comb.cu).  NCW consumer warps + 1 producer warp.  A consumer lane is
 // (chain c = lane % G, worker q = lane / G); worker w = warp * (32/G) + q takes block w of every
 // chunk of CB = NCW*32/G blocks.  The producer (copy) warp streams the J runs of j and k, chunk by chunk,
-// into a ring of NST stages, and fills one slot per update of a second ring (kBD slots): the update's B_jk
-// couplings (FP32, N >= 48) and the random part of every chain's proposal (8 chains per block).  Work units = (group, run of sweeps) come from a ticket counter; a unit
+// into a ring of NST stages and, with 8 chains per block, draws the random part of every chain's proposal into one
+// slot per update of a second ring (kBD slots).  Work units = (group, run of sweeps) come from a ticket counter; a unit
 // waits (bounded) until the previous run of its group has been written back.
-// Ring depth: as many stages as fit next to the amplitude and window tables of the largest N (up to kNstMax), so
+// Ring depth: as many stages as fit next to the amplitude table of the largest N (up to kNstMax), so
 // that the copies of a chunk are issued several chunks ahead of its use (L2 misses of the coupling runs).
 constexpr int kNstMax = 6, kNstMin = 2;
-// Per-update slots (B_jk couplings for N >= 48 on the FP32 path, proposal draws with 8 chains per block): the copy
-// warp fills an update's slot before it streams the update's coupling runs, up to kBD updates ahead of the field
-// warps.
+// Proposal slots: the copy warp is up to kBD updates ahead of the field warps.
 constexpr int kBD = 4;
 
 template <typename real, int G, int NCW> struct SweepShape {
@@ -440,7 +219,6 @@ template <typename real, int G, int NCW> struct SweepShape {
     static constexpr int NTHREADS = (NCW + 1) * 32;
     static constexpr int JS = JStride<real>::value;
     static constexpr size_t stage_bytes = (size_t)2 * CB * JS * sizeof(real);
-    static constexpr bool PACKED = sizeof(real) == 4;  // packed-FP32 block arithmetic (every FP32 shape)
 };
 
 // Shared memory of the sweep kernel without the coupling ring.
@@ -451,8 +229,6 @@ template <typename real, int G, int NCW> size_t sweep_fixed_bytes(int maxN) {
     b += 2 * (kNstMax + kBD) * sizeof(uint64_t);                          // mbarriers
     b = (b + 127) / 128 * 128;
     b += (size_t)(maxN + 2 * APAD) * Sh::RS * sizeof(V);                  // amplitudes
-    if (Sh::PACKED) b += (size_t)(maxN + 2 * APAD) * G * sizeof(float4);      // window table
-    if (kGatherB<real, G>) b += (size_t)kBD * maxN * sizeof(real);            // gathered B_jk couplings
     b += (size_t)2 * NCW * G * 8 * sizeof(real);                          // reduction, double-buffered
     if (kCopyDraws<G>) b += (size_t)kBD * G * sizeof(ProposalDraw<real>);  // proposal draws of kBD updates
     b += (size_t)2 * G * sizeof(Proposal<real>) + 16;                     // proposals, double-buffered
@@ -479,13 +255,12 @@ template <typename real, int G, int NCW>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams prm) {
     using Sh = SweepShape<real, G, NCW>;
     using V = typename vec2<real>::type;
-    constexpr int RS = Sh::RS, CB = Sh::CB, WPW = Sh::WPW, JS = Sh::JS, NW = Sh::NW;
+    constexpr int RS = Sh::RS, CB = Sh::CB, WPW = Sh::WPW, JS = Sh::JS;
     const int NST = prm.nst;  // ring stages (kNstMin .. kNstMax), chosen by the launcher for the largest N
     constexpr int NCT = NCW * 32;  // consumer threads
-    // decision step (see the end of an update): 16 chains per block spread it over 8 lanes per chain, 32 chains
-    // leave it to warp 0, 8 chains take it redundantly in every warp
+    // decision step (see the end of an update): 16 chains per block spread it over 8 lanes per chain, 8 chains take it
+    // redundantly in every warp
     constexpr bool kSpread = G == 16;
-    constexpr bool kOneDecider = G == 32;
 
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *full = reinterpret_cast<uint64_t *>(smem);
@@ -497,16 +272,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
     off += NST * Sh::stage_bytes;
     V *as = reinterpret_cast<V *>(smem + off);
     off += (size_t)(prm.maxN + 2 * APAD) * RS * sizeof(V);
-    float4 *awin = nullptr;
-    if (Sh::PACKED) {
-        awin = reinterpret_cast<float4 *>(smem + off);
-        off += (size_t)(prm.maxN + 2 * APAD) * G * sizeof(float4);
-    }
-    real *bvals = nullptr;  // [kBD][maxN]: B_jk couplings of an update, s = max(j,k) + i
-    if (kGatherB<real, G>) {
-        bvals = reinterpret_cast<real *>(smem + off);
-        off += (size_t)kBD * prm.maxN * sizeof(real);
-    }
     real *red = reinterpret_cast<real *>(smem + off);
     off += (size_t)2 * NCW * G * 8 * sizeof(real);
     off = (off + 15) / 16 * 16;
@@ -600,8 +365,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
         const SampleDev sd = prm.samples[gr.sample];
         const int N = sd.N;
         const int sw0 = ci * spu, sw1 = min(n_sweeps, sw0 + spu);
-        const bool gatherB = kGatherB<real, G> && N >= kGatherBMinN;
-        const bool useSlot = kCopyDraws<G> || gatherB;  // the copy warp fills a slot for every update
+        constexpr bool useSlot = kCopyDraws<G>;  // the copy warp fills a slot for every update
 
         // ---- unit set-up: tables, chain metadata, amplitudes (consumers); producer starts streaming
         if (!producer) {
@@ -626,28 +390,17 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                 V v; v.x = v.y = real(0);
                 if (x >= 0 && x < N && cc < gr.count) {
                     const V *src = A + sd.a_off + (int64_t)(gr.chain0 - sd.chain0 + cc) * N + x;
-                    if (sizeof(real) == 4) {
-                        const float2 t = __ldcg(reinterpret_cast<const float2 *>(src));
-                        v.x = (real)t.x; v.y = (real)t.y;
-                    } else {
-                        const double2 t = __ldcg(reinterpret_cast<const double2 *>(src));
-                        v.x = (real)t.x; v.y = (real)t.y;
-                    }
+                    const double2 t = __ldcg(reinterpret_cast<const double2 *>(src));
+                    v.x = (real)t.x; v.y = (real)t.y;
                 }
                 as[(x + APAD) * RS + cc] = v;
             }
             named_bar(1, NCT);
-            if (Sh::PACKED) {
-                for (int i = tid; i < rows * G; i += NCT)
-                    packed_rows<RS>(reinterpret_cast<const float2 *>(as), awin, G, i / G, rows, i % G);
-                named_bar(1, NCT);
-            }
         }
 
         if (producer) {
             // ---------------- producer warp: stream J runs of (j,k) for every update of the unit
             const int *bo_g = prm.bo + sd.tab_off;
-            const int *xtlo_g = prm.xtlo + sd.tab_off;
             // identity of chain `lane` of the group (the Philox stream of its proposals): (sample, replica,
             // temperature index its slot holds)
             uint32_t pid = 0u;
@@ -674,12 +427,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                         if (mbar_wait_bounded(&bempty[slot], bph ^ 1u, prm.ctl, 4, abort_flag)) {
                             if (kCopyDraws<G> && lane < gr.count)
                                 pdraw[slot * G + lane] = draw_proposal<real>(prm.seed, pid, sweep, (uint32_t)u);
-                            if (kGatherB<real, G> && gatherB) {
-                                const int sB0 = max(j, k), nB = min(j, k) + N - sB0;
-                                real *bv = bvals + (size_t)slot * prm.maxN;
-                                for (int i = lane; i < nB; i += 32)
-                                    bv[i] = b_coupling<real>(J, bo_g, xtlo_g, Rg, sB0 + i, k);
-                            }
                         }
                         mbar_arrive(&bfull[slot]);
                     }
@@ -750,8 +497,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                     }
                     Partials<real> pr;
                     pr.zero();
-                    PartialsX2 prx;
-                    prx.zero();
                     for (int cb = Rg.ulo; cb < Rg.uhi; cb += CB, ++q, rph ^= (++rst == NST) ? 1u : 0u, rst = (rst == NST) ? 0 : rst) {
                         const int stage = rst;
                         const uint32_t ph = rph;
@@ -765,37 +510,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                             const int mode = ((b >= Rg.jlo && b < Rg.jhi) ? 1 : 0) | ((b >= Rg.klo && b < Rg.khi) ? 2 : 0);
                             const real *st_j = ring + (size_t)stage * 2 * CB * JS + (size_t)worker * JS;
                             const real *st_k = st_j + (size_t)CB * JS;
-                            if constexpr (Sh::PACKED) {
-                                const float2 *asf = reinterpret_cast<const float2 *>(as);
-                                const float *fj = reinterpret_cast<const float *>(st_j), *fk = reinterpret_cast<const float *>(st_k);
-                                if (gatherB) process_block_x2_dispatch<G, false>(mode, asf, awin, c, st * TS, xt * TX, j, k, N, fj, fk, prx);
-                                else process_block_x2_dispatch<G, true>(mode, asf, awin, c, st * TS, xt * TX, j, k, N, fj, fk, prx);
-                            } else {
-                                if (gatherB) process_block_dispatch<real, RS, false>(mode, as, c, st * TS, xt * TX, j, k, N, st_j, st_k, pr);
-                                else process_block_dispatch<real, RS, true>(mode, as, c, st * TS, xt * TX, j, k, N, st_j, st_k, pr);
-                            }
+                            process_block_dispatch<real, RS, true>(mode, as, c, st * TS, xt * TX, j, k, N, st_j, st_k, pr);
                         }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&empty[stage]);
-                    }
-                    if constexpr (Sh::PACKED) {
-                        pr.hj.x = prx.hjx.x + prx.hjx.y;
-                        pr.hj.y = (prx.hjy.x + prx.hjy.y) - (prx.hjyn.x + prx.hjyn.y);
-                        pr.hk.x = prx.hkx.x + prx.hkx.y;
-                        pr.hk.y = (prx.hky.x + prx.hky.y) - (prx.hkyn.x + prx.hkyn.y);
-                        pr.B.x = prx.B.x; pr.B.y = prx.B.y;
-                        pr.A.x = prx.A.x; pr.A.y = prx.A.y;
-                    }
-                    // B_jk = sum_s conj(a_{s-j}) J_j[s][{k, s-k}] a_{s-k} over s in [max(j,k), min(j,k)+N) (large N: the
-                    // couplings come from the buffer the copy warp filled; worker w takes s = max(j,k) + w + m NW;
-                    // for smaller N process_block picks them out of the blocks)
-                    if (kGatherB<real, G> && gatherB) {
-                        if (mbar_wait_bounded(&bfull[pslot], pph, prm.ctl, 5, abort_flag)) {
-                            const real *bv = bvals + (size_t)pslot * prm.maxN;
-                            const int sB0 = max(j, k), sB1 = min(j, k) + N;
-                            for (int sb = sB0 + worker; sb < sB1; sb += NW)
-                                caxpy(pr.B, bv[sb - sB0], cmulc(as[(sb - j + APAD) * RS + c], as[(sb - k + APAD) * RS + c]));
-                        }
                     }
                     // every warp is done with the slot (warp 0 copied the proposals out at the update's start)
                     if (useSlot) {
@@ -813,23 +531,9 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                         // layout [warp][chain][value]: the 8 values of one (warp, chain) are consecutive, so that the
                         // reads after the barrier (32 lanes = 4 chains x 8 values of one warp) are 32 consecutive words
                         if (wq == 0) {
-                            if constexpr (sizeof(real) == 4) {
-                                float4 *d = reinterpret_cast<float4 *>(rb + ((size_t)warp * G + c) * 8);
-                                d[0] = make_float4(v[0], v[1], v[2], v[3]);
-                                d[1] = make_float4(v[4], v[5], v[6], v[7]);
-                            } else {
                                 double2 *d = reinterpret_cast<double2 *>(rb + ((size_t)warp * G + c) * 8);
                                 d[0] = make_double2(v[0], v[1]); d[1] = make_double2(v[2], v[3]);
                                 d[2] = make_double2(v[4], v[5]); d[3] = make_double2(v[6], v[7]);
-                            }
-                        }
-                    } else if constexpr (Sh::PACKED) {
-                        // layout [half][warp][chain] of float4: the chains of one (half, warp) are consecutive, so
-                        // the stores and the reads after the barrier are free of bank conflicts
-                        float4 *rb4 = reinterpret_cast<float4 *>(rb);
-                        if (wq == 0) {
-                            rb4[(0 * NCW + warp) * G + c] = make_float4(v[0], v[1], v[2], v[3]);
-                            rb4[(1 * NCW + warp) * G + c] = make_float4(v[4], v[5], v[6], v[7]);
                         }
                     } else {
                         // layout [e][warp][chain]: the 8 chains of one (e, warp) are consecutive words, so both the
@@ -840,38 +544,17 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                             for (int e = 0; e < 8; ++e) rb[(e * NCW + warp) * G + c] = v[e];
                         }
                     }
-                    // packed: the neighbours of j and k for the window rows rewritten on acceptance (modes other
-                    // than j and k keep their values during this update)
-                    float2 nb[4];
-                    if (Sh::PACKED && !kSpread && (!kOneDecider || warp == 0)) {
-                        const float2 *asf = reinterpret_cast<const float2 *>(as);
-                        nb[0] = asf[(j - 1 + APAD) * RS + c]; nb[1] = asf[(j + 1 + APAD) * RS + c];
-                        nb[2] = asf[(k - 1 + APAD) * RS + c]; nb[3] = asf[(k + 1 + APAD) * RS + c];
-                    }
                     named_bar(1, NCT);
-                    // Decision (measured on GB300, per shape):
+                    // Decision:
                     // - 16 chains per block: 8 lanes per chain, 4 chains per warp, warps in turn.  Lane e of a
                     //   chain's group adds value e over the warps in warp order; the group's first lane gathers
-                    //   the 8 totals, decides and writes (+3.7% over warp 0 alone at N = 64);
-                    // - 32 chains per block: warp 0 alone forms the totals, decides and writes (every other warp
-                    //   would repeat the same reads of all partial sums: NCW x G x 8 words each; the 8-lane
-                    //   groups measured 1.5% slower here);
+                    //   the 8 totals, decides and writes; a second barrier orders the writes before the next update;
                     // - 8 chains per block: every warp forms the same totals in the same order, takes the same
-                    //   decision and writes the same values, with no second barrier (measured faster at N = 256).
-                    // With one or more deciding warps a second barrier orders their writes before every warp's next
-                    // update.
+                    //   decision and writes the same values, with no second barrier.
                     if constexpr (kSpread) {
                         for (int c4 = warp * 4; c4 < G; c4 += NCW * 4) {  // warp-uniform trip count
                             const int cd = c4 + (lane >> 3), e = lane & 7;
                             const bool mine = cd < G, lead = mine && e == 0;
-                            // packed: the neighbours of j and k for the window rows rewritten on acceptance (modes
-                            // other than j and k keep their values during this update)
-                            float2 nbs[4];
-                            if (Sh::PACKED && lead) {
-                                const float2 *asf = reinterpret_cast<const float2 *>(as);
-                                nbs[0] = asf[(j - 1 + APAD) * RS + cd]; nbs[1] = asf[(j + 1 + APAD) * RS + cd];
-                                nbs[2] = asf[(k - 1 + APAD) * RS + cd]; nbs[3] = asf[(k + 1 + APAD) * RS + cd];
-                            }
                             real s = 0;
                             if (mine) {
 #pragma unroll
@@ -894,15 +577,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                                 if (acc) {
                                     as[(j + APAD) * RS + cd] = P.nj;
                                     as[(k + APAD) * RS + cd] = P.nk;
-                                    if constexpr (Sh::PACKED) {
-                                        const float2 nj = P.nj, nk = P.nk;
-                                        const float2 jm = (j - 1 == k) ? nk : nbs[0], jp = (j + 1 == k) ? nk : nbs[1];
-                                        const float2 km = (k - 1 == j) ? nj : nbs[2], kp = (k + 1 == j) ? nj : nbs[3];
-                                        awin[(j - 1 + APAD) * G + cd] = make_float4(jm.x, nj.x, jm.y, nj.y);
-                                        awin[(j + APAD) * G + cd] = make_float4(nj.x, jp.x, nj.y, jp.y);
-                                        awin[(k - 1 + APAD) * G + cd] = make_float4(km.x, nk.x, km.y, nk.y);
-                                        awin[(k + APAD) * G + cd] = make_float4(nk.x, kp.x, nk.y, kp.y);
-                                    }
                                 }
                                 if (live) {
                                     if (acc) { cE[cd] += (double)dH; cAcc[cd] += 1u; }
@@ -910,7 +584,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                                 }
                             }
                         }
-                    } else if (!kOneDecider || warp == 0) {
+                    } else {
                         // lane (c, wq) adds the partials of warps wq, wq + WPW, ...: the trip count is the
                         // same on every lane (predicated body), so the warp is converged at the shuffles
                         real t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -918,15 +592,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                         for (int w0 = 0; w0 < NCW; w0 += WPW) {
                             const int w = w0 + wq;
                             if (w < NCW) {
-                                if constexpr (Sh::PACKED) {
-                                    const float4 *rb4 = reinterpret_cast<const float4 *>(rb);
-                                    const float4 lo = rb4[(0 * NCW + w) * G + c], hi = rb4[(1 * NCW + w) * G + c];
-                                    t[0] += lo.x; t[1] += lo.y; t[2] += lo.z; t[3] += lo.w;
-                                    t[4] += hi.x; t[5] += hi.y; t[6] += hi.z; t[7] += hi.w;
-                                } else {
 #pragma unroll
-                                    for (int e = 0; e < 8; ++e) t[e] += rb[(e * NCW + w) * G + c];
-                                }
+                                for (int e = 0; e < 8; ++e) t[e] += rb[(e * NCW + w) * G + c];
                             }
                         }
                         __syncwarp();
@@ -947,17 +614,6 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                             if (acc) {
                                 as[(j + APAD) * RS + c] = P.nj;
                                 as[(k + APAD) * RS + c] = P.nk;
-                                if constexpr (Sh::PACKED) {
-                                    // the window rows j-1, j, k-1, k from registers: row R holds (a_R, a_{R+1});
-                                    // a neighbour that is the other updated mode takes its new value
-                                    const float2 nj = P.nj, nk = P.nk;
-                                    const float2 jm = (j - 1 == k) ? nk : nb[0], jp = (j + 1 == k) ? nk : nb[1];
-                                    const float2 km = (k - 1 == j) ? nj : nb[2], kp = (k + 1 == j) ? nj : nb[3];
-                                    awin[(j - 1 + APAD) * G + c] = make_float4(jm.x, nj.x, jm.y, nj.y);
-                                    awin[(j + APAD) * G + c] = make_float4(nj.x, jp.x, nj.y, jp.y);
-                                    awin[(k - 1 + APAD) * G + c] = make_float4(km.x, nk.x, km.y, nk.y);
-                                    awin[(k + APAD) * G + c] = make_float4(nk.x, kp.x, nk.y, kp.y);
-                                }
                             }
                             if (warp == 0 && c < gr.count) {
                                 if (acc) { cE[c] += (double)dH; cAcc[c] += 1u; }
@@ -966,7 +622,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) sweep_kernel(SweepParams pr
                         }
                     }
                     red_par ^= 1;
-                    if constexpr (kOneDecider || kSpread) named_bar(1, NCT);
+                    if constexpr (kSpread) named_bar(1, NCT);
                     else __syncwarp();
                 }
                 // interior measurement point: snapshot amplitudes and energies
@@ -1235,9 +891,6 @@ static int occupancy_t(int maxN) {
 }
 
 #define PT_SWEEP_VARIANTS(X)                                          \
-    X(float, 8, 7) X(float, 8, 11) X(float, 8, 15)                    \
-    X(float, 16, 7) X(float, 16, 11) X(float, 16, 15)                 \
-    X(float, 32, 3) X(float, 32, 7) X(float, 32, 9) X(float, 32, 11)  \
     X(double, 8, 7) X(double, 16, 3)
 
 bool sweep_variant_exists(bool dbl, int G, int ncw) {
