@@ -3,11 +3,13 @@
 // sweep-segment scheduler (sweeps -> resync -> measure -> swap, replayed as CUDA graphs),
 // checkpoints and the host watchdog.  The declarations and their contracts are in include/pt.h.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 #include <thread>
 #include <tuple>
@@ -211,6 +213,9 @@ struct pt_ctx {
     int4 *d_quads = nullptr;
     int4 *d_rec = nullptr;     // incidence records of the FP32 quadruplet-list path
     float *d_recJ = nullptr;
+    int4 *d_chunks = nullptr, *d_cross = nullptr;  // lists of the pair-table graph sweep
+    int *d_choff = nullptr, *d_xoff = nullptr;
+    int max_chunks = 0, max_cross = 0;
     double *d_Jq = nullptr;
     int *d_inc_off = nullptr, *d_inc = nullptr;
     int G = 8, ncw = 8, spu = 1, grid = 1;
@@ -313,8 +318,10 @@ int cluster_blocks(int G, int ncw, int maxN, int groups, int sms) {
 
 GraphParams graph_params(pt_ctx *c) {
     GraphParams p{};
-    p.samples = c->d_samples; p.groups = c->d_groups; p.quads = c->d_quads; p.Jd = c->d_Jq;
+    p.samples = c->d_samples; p.groups = c->d_groups; p.chain_sample = c->d_chain_sample; p.quads = c->d_quads; p.Jd = c->d_Jq;
     p.inc_off = c->d_inc_off; p.max_deg = c->max_deg; p.rec = c->d_rec; p.recJ = c->d_recJ;
+    p.chunks = c->d_chunks; p.cross = c->d_cross; p.choff = c->d_choff; p.xoff = c->d_xoff;
+    p.max_chunks = c->max_chunks; p.max_cross = c->max_cross;
     p.a = reinterpret_cast<float2 *>(c->d_a);
     p.E = c->d_E; p.label = c->d_label; p.beta = c->d_beta; p.mc_acc = c->d_mc_acc; p.mc_att = c->d_mc_att;
     p.R = c->R; p.nT = c->nT; p.maxN = c->maxN; p.seed = c->seed; p.cc = c->cfg.cc_factor; p.ctl = c->d_ctl;
@@ -777,6 +784,95 @@ void incidence_records(int N, const int32_t *abcd, const double *J, const int *o
         }
 }
 
+// f(s) for every sample, over the host's cores.  False when a call ran out of memory.
+template <typename F> bool for_samples(int S, F &&f) {
+    std::atomic<int> next{0};
+    std::atomic<bool> ok{true};
+    auto work = [&]() {
+        try {
+            for (int s = next++; s < S; s = next++) f(s);
+        } catch (const std::bad_alloc &) {
+            ok = false;
+        }
+    };
+    std::vector<std::thread> pool;
+    const int n = std::min({S, 16, std::max(1, (int)std::thread::hardware_concurrency())});
+    try {
+        pool.reserve(n);
+        for (int i = 1; i < n; ++i) pool.emplace_back(work);
+    } catch (const std::exception &) {  // no more threads: the ones there are, and this one, do the work
+    }
+    work();
+    for (auto &t : pool) t.join();
+    return ok;
+}
+
+// Lists of the pair-table graph sweep, from the incidence records.  chunks: per mode the records grouped by their
+// conjugated partner C (in mode order, list order within) in fours, {pair indices of (A, B), C, 0} and four couplings,
+// padded with zero couplings.  cross: per pair of modes lo < hi the quadruplets that hold both: {the other two modes,
+// conjugation flags of (lo, hi, x, y), J}.
+struct GraphLists {
+    std::vector<int4> chunks, cross;
+    std::vector<int> choff, xoff;
+    int max_chunks = 0, max_cross = 0;
+};
+int4 bits4(float a, float b, float c, float d) {
+    int4 r;
+    std::memcpy(&r.x, &a, 4); std::memcpy(&r.y, &b, 4); std::memcpy(&r.z, &c, 4); std::memcpy(&r.w, &d, 4);
+    return r;
+}
+void graph_lists(int N, int64_t nq, const int32_t *abcd, const double *J, const int *off, const int4 *rec, const float *recJ, GraphLists &g) {
+    auto tri = [N](int x, int y) {
+        const int lo = std::min(x, y), hi = std::max(x, y);
+        return lo * (2 * N - lo - 1) / 2 + hi - lo - 1;
+    };
+    const int RS = ptgb::kGraphRowStride;
+    g.choff.assign(N + 1, 0);
+    std::vector<std::vector<int>> by(N);
+    for (int l = 0; l < N; ++l) {
+        for (auto &v : by) v.clear();
+        for (int e = off[l]; e < off[l + 1]; ++e) by[rec[e].z / RS].push_back(e);
+        for (int C = 0; C < N; ++C)
+            for (size_t i = 0; i < by[C].size(); i += 4) {
+                unsigned pi[4] = {0, 0, 0, 0};
+                float jv[4] = {0.f, 0.f, 0.f, 0.f};
+                for (size_t m = i; m < std::min(i + 4, by[C].size()); ++m) {
+                    pi[m - i] = (unsigned)tri(rec[by[C][m]].x / RS, rec[by[C][m]].y / RS);
+                    jv[m - i] = recJ[by[C][m]];
+                }
+                g.chunks.push_back(make_int4((int)(pi[0] | pi[1] << 16), (int)(pi[2] | pi[3] << 16), C, 0));
+                g.chunks.push_back(bits4(jv[0], jv[1], jv[2], jv[3]));
+            }
+        g.choff[l + 1] = (int)(g.chunks.size() / 2);
+        g.max_chunks = std::max(g.max_chunks, g.choff[l + 1] - g.choff[l]);
+    }
+    const int np = N * (N - 1) / 2;
+    g.xoff.assign(np + 1, 0);
+    for (int64_t q = 0; q < nq; ++q)
+        for (int a = 0; a < 4; ++a)
+            for (int b = a + 1; b < 4; ++b) g.xoff[tri(abcd[4 * q + a], abcd[4 * q + b]) + 1]++;
+    for (int i = 0; i < np; ++i) {
+        g.max_cross = std::max(g.max_cross, g.xoff[i + 1]);
+        g.xoff[i + 1] += g.xoff[i];
+    }
+    g.cross.resize(g.xoff[np]);
+    std::vector<int> fill(g.xoff.begin(), g.xoff.end() - 1);
+    for (int64_t q = 0; q < nq; ++q)
+        for (int a = 0; a < 4; ++a)
+            for (int b = a + 1; b < 4; ++b) {
+                const int32_t *m = abcd + 4 * q;
+                const int lo = m[a] < m[b] ? a : b, hi = a + b - lo;
+                int o[2], n = 0;
+                for (int e = 0; e < 4; ++e)
+                    if (e != a && e != b) o[n++] = e;
+                auto conj = [](int pos) { return pos == 0 || pos == 3 ? 1 : 0; };
+                int4 x = bits4(0.f, 0.f, 0.f, (float)J[q]);
+                x.x = m[o[0]]; x.y = m[o[1]];
+                x.z = conj(lo) | conj(hi) << 1 | conj(o[0]) << 2 | conj(o[1]) << 3;
+                g.cross[fill[tri(m[a], m[b])]++] = x;
+            }
+}
+
 void free_all(pt_ctx *c) {
     drop_graphs(c);
     for (auto &p : c->allocs) {
@@ -1170,7 +1266,8 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         std::vector<int> hinc_off, hinc((size_t)std::max<int64_t>(inc_total, 1));
         std::vector<int4> hrec(c->gfp32 ? hinc.size() : 0);
         std::vector<float> hrecJ(c->gfp32 ? hinc.size() : 0);
-        for (int s = 0; s < S; ++s) {
+        std::vector<std::vector<int>> offs(S);
+        auto build = [&](int s) {
             const int n = c->N[s];
             const SampleDev &sd = c->samples[s];
             std::vector<int32_t> abcd((size_t)4 * std::max<int64_t>(sd.nq, 1));
@@ -1181,13 +1278,48 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
                 hq[sd.q_off + q] = make_int4(abcd[4 * q], abcd[4 * q + 1], abcd[4 * q + 2], abcd[4 * q + 3]);
                 hJq[sd.q_off + q] = J[J_offsets[s] + q];
             }
-            std::vector<int> off(n + 1);
-            incidence_lists(n, cnt, abcd.data(), off.data(), hinc.data() + sd.inc_off);
-            for (int l = 0; l < n; ++l) c->max_deg = std::max(c->max_deg, off[l + 1] - off[l]);
-            hinc_off.insert(hinc_off.end(), off.begin(), off.end());
+            offs[s].resize(n + 1);
+            incidence_lists(n, cnt, abcd.data(), offs[s].data(), hinc.data() + sd.inc_off);
             if (c->gfp32)
-                incidence_records(n, abcd.data(), J + J_offsets[s], off.data(), hinc.data() + sd.inc_off,
+                incidence_records(n, abcd.data(), J + J_offsets[s], offs[s].data(), hinc.data() + sd.inc_off,
                                   hrec.data() + sd.inc_off, hrecJ.data() + sd.inc_off);
+        };
+        if (!for_samples(S, build)) return bail(fail(c, PT_ENOMEM, "host allocation failed (quadruplet lists)"));
+        for (int s = 0; s < S; ++s) {
+            for (int l = 0; l < c->N[s]; ++l) c->max_deg = std::max(c->max_deg, offs[s][l + 1] - offs[s][l]);
+            hinc_off.insert(hinc_off.end(), offs[s].begin(), offs[s].end());
+        }
+        if (c->gfp32 && graph_table_candidate(c->maxN, c->max_deg)) {
+            std::vector<GraphLists> lists(S);
+            auto make = [&](int s) {
+                const SampleDev &sd = c->samples[s];
+                graph_lists(c->N[s], sd.nq, graph + 4 * J_offsets[s], J + J_offsets[s], offs[s].data(), hrec.data() + sd.inc_off,
+                            hrecJ.data() + sd.inc_off, lists[s]);
+            };
+            if (!for_samples(S, make)) return bail(fail(c, PT_ENOMEM, "host allocation failed (graph lists)"));
+            int64_t nch = 0, ncr = 0, nco = 0, nxo = 0;
+            for (int s = 0; s < S; ++s) {
+                SampleDev &sd = c->samples[s];
+                sd.chunk_off = nch / 2; sd.cross_off = ncr; sd.xoff_off = nxo;
+                nch += (int64_t)lists[s].chunks.size(); ncr += (int64_t)lists[s].cross.size();
+                nco += (int64_t)lists[s].choff.size(); nxo += (int64_t)lists[s].xoff.size();
+                c->max_chunks = std::max(c->max_chunks, lists[s].max_chunks);
+                c->max_cross = std::max(c->max_cross, lists[s].max_cross);
+            }
+            RC(dalloc(c, &c->d_chunks, nch));
+            RC(dalloc(c, &c->d_cross, ncr));
+            RC(dalloc(c, &c->d_choff, nco));
+            RC(dalloc(c, &c->d_xoff, nxo));
+            nco = 0;
+            for (int s = 0; s < S; ++s) {
+                const SampleDev &sd = c->samples[s];
+                const GraphLists &g = lists[s];
+                CK(cudaMemcpy(c->d_chunks + 2 * sd.chunk_off, g.chunks.data(), g.chunks.size() * sizeof(int4), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_cross + sd.cross_off, g.cross.data(), g.cross.size() * sizeof(int4), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_choff + nco, g.choff.data(), g.choff.size() * sizeof(int), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_xoff + sd.xoff_off, g.xoff.data(), g.xoff.size() * sizeof(int), cudaMemcpyHostToDevice));
+                nco += (int64_t)g.choff.size();
+            }
         }
         RC(dalloc(c, &c->d_quads, hq.size()));
         RC(dalloc(c, &c->d_Jq, hJq.size()));
@@ -1238,7 +1370,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemset(c->d_qstat, 0, (size_t)S * n_T * PT_NQSTAT * sizeof(double)));
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
 
-    if (c->gfp32) CK(graph_prepare(c->maxN, c->max_deg));
+    if (c->gfp32) CK(graph_prepare(graph_params(c)));
     if (c->row) {
         c->d_Jrow = dev_alloc(c, (size_t)row_total * c->esize);
         if (!c->d_Jrow) return bail(fail(c, PT_ENOMEM, "device allocation failed (couplings)"));

@@ -137,6 +137,7 @@ constexpr int kGraphRowStride = 8;
 
 struct GraphParams {
     const SampleDev *samples;
+    const int *chain_sample; // chain slot -> sample
     const GroupDev *groups;
     const int4 *quads;       // quadruplets in term order, per sample at q_off (energy kernel)
     const double *Jd;        // FP64 couplings (energy kernel)
@@ -147,6 +148,12 @@ struct GraphParams {
     // record's own mode | positions of A, B, C << 2, 4, 6
     const int4 *rec;
     const float *recJ;       // coupling of each incidence record
+    // pair-table sweep (null when not built): chunks of four records per mode (two int4 each: pair indices, partner; then
+    // four couplings), their offsets per mode (N+1, at mode_off), and per pair of modes the quadruplets that hold both
+    const int4 *chunks, *cross;
+    const int *choff, *xoff;
+    int max_chunks, max_cross;  // largest lists of one mode / one pair
+    int tab_nbuf;               // list buffers (set by the launcher)
     float2 *a;
     double *E;
     const int *label;
@@ -169,7 +176,8 @@ struct GraphParams {
 cudaError_t launch_wait_probe(Control *ctl, unsigned long long limit_ns, cudaStream_t s);
 cudaError_t launch_graph_sweep(const GraphParams &p, int n_groups, cudaStream_t s);
 cudaError_t launch_graph_energy(const GraphParams &p, int n_groups, cudaStream_t s);
-cudaError_t graph_prepare(int maxN, int max_deg);  // shared-memory limits of the graph kernels (N <= maxN)
+cudaError_t graph_prepare(const GraphParams &p);      // shared-memory limits of the kernels it takes
+bool graph_table_candidate(int maxN, int max_deg);
 
 // pt_row.cu: one chain per block, pair products resident in shared memory (FP64, and FP32 at small N)
 constexpr int kRowMaxThreads = 352;  // N <= 160: ten row warps and the helper
