@@ -57,6 +57,34 @@ cudaError_t launch_init(const InitParams &p, int n_chains, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------------------------------------
+// Canonical order: chain slot -> (sample, replica, temperature its label names).  One warp per chain.
+template <typename V>
+__global__ void canon_kernel(const SampleDev *samples, const int *chain_sample, const int *label, int nT, const V *a, double2 *a_out,
+                             int64_t lo, int64_t hi, const double *E, double *E_out, int n_chains) {
+    const int slot = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (slot >= n_chains) return;
+    const SampleDev sd = samples[chain_sample[slot]];
+    const int at = (slot - sd.chain0) / nT * nT + label[slot];
+    if (E && lane == 0) E_out[sd.chain0 + at] = E[slot];
+    if (!a) return;
+    const V *src = a + sd.a_off + (int64_t)(slot - sd.chain0) * sd.N;
+    const int64_t dst = sd.a_off + (int64_t)at * sd.N;
+    for (int x = lane; x < sd.N; x += 32) {
+        if (dst + x < lo || dst + x >= hi) continue;
+        const V v = src[x];
+        a_out[dst + x - lo] = make_double2((double)v.x, (double)v.y);
+    }
+}
+
+cudaError_t launch_canon(const SampleDev *samples, const int *chain_sample, const int *label, int nT, const void *a, bool dbl,
+                         double2 *a_out, int64_t lo, int64_t hi, const double *E, double *E_out, int n_chains, cudaStream_t s) {
+    const int grid = (n_chains + 7) / 8;
+    if (dbl) canon_kernel<double2><<<grid, 256, 0, s>>>(samples, chain_sample, label, nT, (const double2 *)a, a_out, lo, hi, E, E_out, n_chains);
+    else canon_kernel<float2><<<grid, 256, 0, s>>>(samples, chain_sample, label, nT, (const float2 *)a, a_out, lo, hi, E, E_out, n_chains);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------------------------------------
 // One swap pass: per (sample, replica) ladder, sequentially i = 0 .. nT-2 (ascending T), exchange the
 // temperatures of the chains at i and i+1 with probability min[1, exp((b_i - b_{i+1})(E_i - E_{i+1}))]
 // (paper Eq. (15)).  Labels are exchanged instead of configurations.  The per-chain Metropolis

@@ -202,6 +202,8 @@ struct pt_ctx {
     void *d_a = nullptr;
     double *d_E = nullptr, *d_beta = nullptr, *d_Etmp = nullptr;
     int *d_label = nullptr, *d_perm = nullptr, *d_chain_sample = nullptr, *d_progress = nullptr;
+    unsigned long long *d_acc = nullptr;  // all accumulators (the pointers below lie in it)
+    size_t acc_words = 0;
     unsigned long long *d_mc_acc = nullptr, *d_mc_att = nullptr, *d_mcT_acc = nullptr, *d_mcT_att = nullptr;
     unsigned long long *d_swap_acc = nullptr, *d_swap_att = nullptr, *d_qhist = nullptr;
     double *d_stat = nullptr, *d_qstat = nullptr, *d_fields = nullptr;
@@ -273,6 +275,8 @@ template <typename T> int upload(pt_ctx *c, T *dst, const T *src, size_t count) 
     return PT_OK;
 }
 
+constexpr size_t kAccStaged = 64 * 1024;  // accumulator words (8 bytes) that pt_measure brings out in one copy
+
 int watchdog_sync(pt_ctx *c) {
     const auto t0 = std::chrono::steady_clock::now();
     for (;;) {
@@ -283,7 +287,9 @@ int watchdog_sync(pt_ctx *c) {
             const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
             if (ms > c->cfg.watchdog_ms) return fail(c, PT_ETIMEOUT, "host watchdog: stream did not finish in time");
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        // short waits poll (a sleep takes 50 us and more to return), long ones leave the core to others
+        if (std::chrono::steady_clock::now() - t0 < std::chrono::milliseconds(2)) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
     Control h;
     CK(cudaMemcpy(&h, c->d_ctl, sizeof(Control), cudaMemcpyDeviceToHost));
@@ -1233,18 +1239,21 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     RC(dalloc(c, &c->d_perm, c->n_chains));
     RC(dalloc(c, &c->d_chain_sample, c->n_chains));
     RC(dalloc(c, &c->d_progress, c->max_groups));
-    RC(dalloc(c, &c->d_mc_acc, c->n_chains));
-    RC(dalloc(c, &c->d_mc_att, c->n_chains));
-    RC(dalloc(c, &c->d_mcT_acc, (size_t)S * n_T));
-    RC(dalloc(c, &c->d_mcT_att, (size_t)S * n_T));
-    RC(dalloc(c, &c->d_gm_acc, (size_t)S * n_T));
-    RC(dalloc(c, &c->d_gm_att, (size_t)S * n_T));
-    const size_t npair = (size_t)S * replicas * std::max(1, n_T - 1);
-    RC(dalloc(c, &c->d_swap_acc, npair));
-    RC(dalloc(c, &c->d_swap_att, npair));
-    RC(dalloc(c, &c->d_qhist, (size_t)S * n_T * PT_QBINS));
-    RC(dalloc(c, &c->d_stat, (size_t)S * n_T * PT_NSTAT));
-    RC(dalloc(c, &c->d_qstat, (size_t)S * n_T * PT_NQSTAT));
+    // all accumulators in one block of 8-byte words: one copy brings them out, one memset clears them
+    const size_t npair = (size_t)S * replicas * std::max(1, n_T - 1), ST = (size_t)S * n_T;
+    c->acc_words = ST * (PT_NSTAT + PT_NQSTAT + PT_QBINS + 4) + 2 * npair + 2 * (size_t)c->n_chains;
+    RC(dalloc(c, &c->d_acc, c->acc_words));
+    {
+        unsigned long long *w = c->d_acc;
+        auto take = [&](size_t n) { unsigned long long *at = w; w += n; return at; };
+        c->d_stat = reinterpret_cast<double *>(take(ST * PT_NSTAT));
+        c->d_qstat = reinterpret_cast<double *>(take(ST * PT_NQSTAT));
+        c->d_qhist = take(ST * PT_QBINS);
+        c->d_swap_acc = take(npair); c->d_swap_att = take(npair);
+        c->d_gm_acc = take(ST); c->d_gm_att = take(ST);
+        c->d_mcT_acc = take(ST); c->d_mcT_att = take(ST);
+        c->d_mc_acc = take(c->n_chains); c->d_mc_att = take(c->n_chains);
+    }
     RC(dalloc(c, &c->d_fields, (size_t)chains_ps * 8));
     RC(dalloc(c, &c->d_ctl, 1));
 
@@ -1357,17 +1366,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemcpy(c->d_perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_chain_sample, c->chain_sample.data(), c->chain_sample.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_beta, beta.data(), n_T * sizeof(double), cudaMemcpyHostToDevice));
-    CK(cudaMemset(c->d_mc_acc, 0, c->n_chains * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_mc_att, 0, c->n_chains * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_mcT_acc, 0, (size_t)S * n_T * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_mcT_att, 0, (size_t)S * n_T * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_gm_acc, 0, (size_t)S * n_T * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_gm_att, 0, (size_t)S * n_T * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_swap_acc, 0, npair * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_swap_att, 0, npair * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_qhist, 0, (size_t)S * n_T * PT_QBINS * sizeof(unsigned long long)));
-    CK(cudaMemset(c->d_stat, 0, (size_t)S * n_T * PT_NSTAT * sizeof(double)));
-    CK(cudaMemset(c->d_qstat, 0, (size_t)S * n_T * PT_NQSTAT * sizeof(double)));
+    CK(cudaMemset(c->d_acc, 0, c->acc_words * sizeof(unsigned long long)));
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
 
     if (c->gfp32) CK(graph_prepare(graph_params(c)));
@@ -1473,25 +1472,44 @@ int pt_measure_now(pt_ctx *c) {
     return run_measure(c, 0, 1);
 }
 
+// Writes to a page fault it in; the byte keeps its value.  Faulting the pages of a fresh host buffer in here, while the
+// device still works, is several times cheaper than letting the copy engine do it (4 MB: 55 us against 190).
+static void touch_pages(void *p, size_t bytes) {
+    volatile char *q = reinterpret_cast<char *>(p);
+    for (size_t i = 0; i < bytes; i += 4096) q[i] = q[i];
+}
+
 int pt_measure(pt_ctx *c, pt_observables *o) {
     if (!c || !o) return fail(c, PT_EINVAL, "pt_measure: NULL argument");
     int rc = watchdog_sync(c);
     if (rc != PT_OK) return rc;
     const size_t ST = (size_t)c->S * c->nT, npair = (size_t)c->S * c->R * std::max(1, c->nT - 1);
-    if (o->stat) CK(cudaMemcpy(o->stat, c->d_stat, ST * PT_NSTAT * sizeof(double), cudaMemcpyDeviceToHost));
-    if (o->qstat) CK(cudaMemcpy(o->qstat, c->d_qstat, ST * PT_NQSTAT * sizeof(double), cudaMemcpyDeviceToHost));
-    if (o->qhist) CK(cudaMemcpy(o->qhist, c->d_qhist, ST * PT_QBINS * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-    if (o->swap_acc) CK(cudaMemcpy(o->swap_acc, c->d_swap_acc, npair * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-    if (o->swap_att) CK(cudaMemcpy(o->swap_att, c->d_swap_att, npair * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-    if (o->gm_acc) CK(cudaMemcpy(o->gm_acc, c->d_gm_acc, ST * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-    if (o->gm_att) CK(cudaMemcpy(o->gm_att, c->d_gm_att, ST * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+    // small accumulators come in one copy and are handed out from it; large ones go straight to the caller
+    std::vector<unsigned long long> all;
+    if (c->acc_words <= kAccStaged) {
+        all.resize(c->acc_words);
+        CK(cudaMemcpy(all.data(), c->d_acc, c->acc_words * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+    }
+    auto get = [&](void *dst, const void *src, size_t words) {
+        if (!dst) return cudaSuccess;
+        if (all.empty()) return cudaMemcpy(dst, src, words * 8, cudaMemcpyDeviceToHost);
+        std::memcpy(dst, all.data() + (reinterpret_cast<const unsigned long long *>(src) - c->d_acc), words * 8);
+        return cudaSuccess;
+    };
+    CK(get(o->stat, c->d_stat, ST * PT_NSTAT));
+    CK(get(o->qstat, c->d_qstat, ST * PT_NQSTAT));
+    CK(get(o->qhist, c->d_qhist, ST * PT_QBINS));
+    CK(get(o->swap_acc, c->d_swap_acc, npair));
+    CK(get(o->swap_att, c->d_swap_att, npair));
+    CK(get(o->gm_acc, c->d_gm_acc, ST));
+    CK(get(o->gm_att, c->d_gm_att, ST));
     if (o->mc_acc || o->mc_att) {
         std::vector<unsigned long long> ta(ST), tt(ST), ca(c->n_chains), ct(c->n_chains);
         std::vector<int> lab(c->n_chains);
-        CK(cudaMemcpy(ta.data(), c->d_mcT_acc, ST * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(tt.data(), c->d_mcT_att, ST * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(ca.data(), c->d_mc_acc, c->n_chains * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(ct.data(), c->d_mc_att, c->n_chains * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+        CK(get(ta.data(), c->d_mcT_acc, ST));
+        CK(get(tt.data(), c->d_mcT_att, ST));
+        CK(get(ca.data(), c->d_mc_acc, c->n_chains));
+        CK(get(ct.data(), c->d_mc_att, c->n_chains));
         CK(cudaMemcpy(lab.data(), c->d_label, c->n_chains * sizeof(int), cudaMemcpyDeviceToHost));
         for (int slot = 0; slot < c->n_chains; ++slot) {
             const size_t i = (size_t)c->chain_sample[slot] * c->nT + lab[slot];
@@ -1506,18 +1524,7 @@ int pt_measure(pt_ctx *c, pt_observables *o) {
 
 int pt_reset_observables(pt_ctx *c) {
     if (!c) return fail(nullptr, PT_EINVAL, "pt_reset_observables: NULL context");
-    const size_t ST = (size_t)c->S * c->nT, npair = (size_t)c->S * c->R * std::max(1, c->nT - 1);
-    CK(cudaMemsetAsync(c->d_stat, 0, ST * PT_NSTAT * sizeof(double), c->stream));
-    CK(cudaMemsetAsync(c->d_qstat, 0, ST * PT_NQSTAT * sizeof(double), c->stream));
-    CK(cudaMemsetAsync(c->d_qhist, 0, ST * PT_QBINS * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_swap_acc, 0, npair * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_swap_att, 0, npair * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_mcT_acc, 0, ST * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_mcT_att, 0, ST * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_mc_acc, 0, c->n_chains * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_mc_att, 0, c->n_chains * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_gm_acc, 0, ST * sizeof(uint64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_gm_att, 0, ST * sizeof(uint64_t), c->stream));
+    CK(cudaMemsetAsync(c->d_acc, 0, c->acc_words * sizeof(unsigned long long), c->stream));
     return PT_OK;
 }
 
@@ -1536,26 +1543,21 @@ static int canonical_map(pt_ctx *c, std::vector<int> &canon) {
 
 int pt_get_state(pt_ctx *c, double *a, double *E) {
     if (!c) return fail(nullptr, PT_EINVAL, "pt_get_state: NULL context");
-    int rc = watchdog_sync(c);
-    if (rc != PT_OK) return rc;
-    std::vector<int> canon;
-    if ((rc = canonical_map(c, canon)) != PT_OK) return rc;
-    if (a) {
-        std::vector<unsigned char> h((size_t)c->a_total * 2 * c->esize);
-        CK(cudaMemcpy(h.data(), c->d_a, h.size(), cudaMemcpyDeviceToHost));
-        for (int slot = 0; slot < c->n_chains; ++slot) {
-            const SampleDev &sd = c->samples[c->chain_sample[slot]];
-            const int64_t src = sd.a_off + (int64_t)(slot - sd.chain0) * sd.N;
-            const int64_t dst = sd.a_off + (int64_t)(canon[slot] - sd.chain0) * sd.N;
-            for (int x = 0; x < 2 * sd.N; ++x)
-                a[2 * dst + x] = c->dbl ? reinterpret_cast<double *>(h.data())[2 * src + x]
-                                        : (double)reinterpret_cast<float *>(h.data())[2 * src + x];
-        }
-    }
-    if (E) {
-        std::vector<double> h(c->n_chains);
-        CK(cudaMemcpy(h.data(), c->d_E, c->n_chains * sizeof(double), cudaMemcpyDeviceToHost));
-        for (int slot = 0; slot < c->n_chains; ++slot) E[canon[slot]] = h[slot];
+    // Amplitudes (widened to FP64) and energies are put in canonical order on the device, so that each is a plain copy.
+    // The snapshots, which hold nothing between segments, serve as the buffer: the state goes through in as many pieces
+    // as that takes (one with two FP32 snapshots or an FP64 one, else two).
+    const int64_t cap = std::max<int64_t>(1, (int64_t)((size_t)c->n_snap_max * c->a_total * 2 * c->esize / sizeof(double2)));
+    double2 *canon = reinterpret_cast<double2 *>(c->d_snap_a);
+    for (int64_t lo = 0; lo == 0 || (a && lo < c->a_total); lo += cap) {
+        const int64_t n = std::min(cap, c->a_total - lo);
+        const bool first = lo == 0;
+        CK(launch_canon(c->d_samples, c->d_chain_sample, c->d_label, c->nT, a ? c->d_a : nullptr, c->dbl, canon, lo, lo + n,
+                        first && E ? c->d_E : nullptr, c->d_snap_E, c->n_chains, c->stream));
+        if (a) touch_pages(a + 2 * lo, (size_t)n * sizeof(double2));
+        const int rc = watchdog_sync(c);
+        if (rc != PT_OK) return rc;
+        if (a) CK(cudaMemcpy(a + 2 * lo, canon, (size_t)n * sizeof(double2), cudaMemcpyDeviceToHost));
+        if (first && E) CK(cudaMemcpy(E, c->d_snap_E, c->n_chains * sizeof(double), cudaMemcpyDeviceToHost));
     }
     return PT_OK;
 }
@@ -1587,12 +1589,10 @@ int pt_energy(pt_ctx *c, double *E) {
     if (!c || !E) return fail(c, PT_EINVAL, "pt_energy: NULL argument");
     int rc = run_energy(c, 0, c->d_Etmp, false);
     if (rc != PT_OK) return rc;
+    CK(launch_canon(c->d_samples, c->d_chain_sample, c->d_label, c->nT, nullptr, c->dbl, nullptr, 0, 0, c->d_Etmp, c->d_snap_E, c->n_chains,
+                    c->stream));
     if ((rc = watchdog_sync(c)) != PT_OK) return rc;
-    std::vector<int> canon;
-    if ((rc = canonical_map(c, canon)) != PT_OK) return rc;
-    std::vector<double> h(c->n_chains);
-    CK(cudaMemcpy(h.data(), c->d_Etmp, c->n_chains * sizeof(double), cudaMemcpyDeviceToHost));
-    for (int slot = 0; slot < c->n_chains; ++slot) E[canon[slot]] = h[slot];
+    CK(cudaMemcpy(E, c->d_snap_E, c->n_chains * sizeof(double), cudaMemcpyDeviceToHost));
     return PT_OK;
 }
 
@@ -1942,6 +1942,7 @@ int pt_learn_params(pt_ctx *c, float *P, int set) {
         if ((rc = learn_cast(c)) != PT_OK) return rc;
         return watchdog_sync(c);
     }
+    touch_pages(P, n * sizeof(float));
     CK(cudaMemcpy(P, L.P, n * sizeof(float), cudaMemcpyDeviceToHost));
     return PT_OK;
 }

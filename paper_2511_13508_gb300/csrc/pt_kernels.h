@@ -238,6 +238,11 @@ struct PlainParams {
 cudaError_t launch_plain_sweep(const PlainParams &p, int n_chains, cudaStream_t s);
 cudaError_t launch_plain_energy(const PlainParams &p, int n_chains, cudaStream_t s);
 
+// Chain state in canonical (sample, replica, temperature) order (a or E may be null): amplitudes widened to FP64, elements
+// [lo, hi) of the canonical state at a_out, and energies.
+cudaError_t launch_canon(const SampleDev *samples, const int *chain_sample, const int *label, int nT, const void *a, bool dbl,
+                         double2 *a_out, int64_t lo, int64_t hi, const double *E, double *E_out, int n_chains, cudaStream_t s);
+
 cudaError_t launch_advance(Control *ctl, long long sweeps, long long swap_passes, long long rounds, cudaStream_t s);
 
 }  // namespace ptgb
