@@ -89,37 +89,66 @@ cudaError_t launch_canon(const SampleDev *samples, const int *chain_sample, cons
 // temperatures of the chains at i and i+1 with probability min[1, exp((b_i - b_{i+1})(E_i - E_{i+1}))]
 // (paper Eq. (15)).  Labels are exchanged instead of configurations.  The per-chain Metropolis
 // counters are first folded into per-temperature counters under the labels they were earned with.
-__global__ void swap_kernel(SwapParams p) {
-    const int ladder = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ladder >= p.S * p.R) return;
-    const int s = ladder / p.R;
+// One warp per ladder.  The sequence is a chain of FP64 operations, so everything else is taken off it: chains, energies
+// and counters are loaded by all lanes, and the uniforms are drawn as log U, a lane each, so that a step is a difference,
+// a product and a comparison (it used to hold an exponential and three dependent loads: 78 us for a ladder of 42
+// temperatures on GB300).
+constexpr int kSwapTile = 256;  // temperatures of a ladder handled at once
+
+__global__ void __launch_bounds__(32) swap_kernel(SwapParams p) {
+    __shared__ double sE[kSwapTile + 1], sB[kSwapTile + 1], sL[kSwapTile];
+    __shared__ int sC[kSwapTile + 1], sS[kSwapTile];
+    const int ladder = blockIdx.x, lane = threadIdx.x, s = ladder / p.R;
     int *perm = p.perm + (int64_t)ladder * p.nT;
-    for (int t = 0; t < p.nT; ++t) {
-        const int slot = perm[t];
-        atomicAdd(p.mcT_acc + (int64_t)s * p.nT + t, p.mc_acc[slot]);
-        atomicAdd(p.mcT_att + (int64_t)s * p.nT + t, p.mc_att[slot]);
-        p.mc_acc[slot] = 0ull;
-        p.mc_att[slot] = 0ull;
-    }
     const uint32_t pass = (uint32_t)p.ctl->swap_passes;
-    for (int i = 0; i + 1 < p.nT; ++i) {
-        const int c0 = perm[i], c1 = perm[i + 1];
-        const double D = (p.beta[i] - p.beta[i + 1]) * (p.E[c0] - p.E[c1]);
-        const u32x4 w = draw(p.seed, (uint32_t)ladder, pass, (uint32_t)i, kTagSwap);
-        const int64_t pi = (int64_t)ladder * (p.nT - 1) + i;
-        p.swap_att[pi] += 1ull;
-        if (D >= 0.0 || u01(w.x) < exp(D)) {
-            perm[i] = c1; perm[i + 1] = c0;
-            p.label[c0] = i + 1; p.label[c1] = i;
-            p.swap_acc[pi] += 1ull;
+    const int64_t pair0 = (int64_t)ladder * (p.nT - 1);
+    for (int i0 = 0; i0 == 0 || i0 + 1 < p.nT; i0 += kSwapTile) {
+        const int n = min(kSwapTile, p.nT - 1 - i0);  // pairs (i, i+1) of this tile
+        for (int i = lane; i <= n; i += 32) {
+            const int slot = perm[i0 + i];
+            sC[i] = slot;
+            sE[i] = p.E[slot];
+            sB[i] = p.beta[i0 + i];
+            if (i < n) sL[i] = log(u01(draw(p.seed, (uint32_t)ladder, pass, (uint32_t)(i0 + i), kTagSwap).x));
+            if (i > 0 || i0 == 0) {  // entry 0 of a later tile is the last of the one before: folded there
+                atomicAdd(p.mcT_acc + (int64_t)s * p.nT + i0 + i, p.mc_acc[slot]);
+                atomicAdd(p.mcT_att + (int64_t)s * p.nT + i0 + i, p.mc_att[slot]);
+                p.mc_acc[slot] = 0ull;
+                p.mc_att[slot] = 0ull;
+            }
         }
+        __syncwarp();
+        if (n > 0) {
+            int c0 = sC[0];
+            double e0 = sE[0];
+            for (int i = 0; i < n; ++i) {
+                const double e1 = sE[i + 1], D = (sB[i] - sB[i + 1]) * (e0 - e1);
+                const bool swap = D >= 0.0 || sL[i] < D;
+                const int c1 = sC[i + 1];
+                // position i keeps the chain that does not move on
+                if (lane == 0) { sC[i] = swap ? c1 : c0; sS[i] = swap; }
+                if (!swap) { c0 = c1; e0 = e1; }
+            }
+            if (lane == 0) sC[n] = c0;
+        }
+        __syncwarp();
+        for (int i = lane; i <= n; i += 32) {
+            perm[i0 + i] = sC[i];
+            p.label[sC[i]] = i0 + i;
+            if (i < n) {
+                p.swap_att[pair0 + i0 + i] += 1ull;
+                if (sS[i]) p.swap_acc[pair0 + i0 + i] += 1ull;
+            }
+        }
+        __syncwarp();
+        __threadfence_block();
     }
 }
 
 cudaError_t launch_swap(const SwapParams &p, cudaStream_t s) {
     const int n = p.S * p.R;
     if (n <= 0 || p.nT < 2) return cudaSuccess;
-    swap_kernel<<<(n + 127) / 128, 128, 0, s>>>(p);
+    swap_kernel<<<n, 32, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -127,66 +156,89 @@ cudaError_t launch_swap(const SwapParams &p, cudaStream_t s) {
 // Measurements of one (sample, temperature) per block over the snapshots and/or the live state:
 // E, E^2 (specific heat, Eq. (21)), Y2, Y4 (Sec. IV.D), I, I^2 per chain; for every replica pair the
 // overlap q = Re sum conj(a^c) a^d / N (Sec. IV.C), its moments and its 201-bin histogram.
-template <typename V>
-__device__ void measure_one(const MeasureParams &p, const V *a, const double *E, int s, int t, double *scratch) {
-    const SampleDev sd = p.samples[s];
-    const int N = sd.N;
-    double *st = p.stat + ((int64_t)s * p.nT + t) * 7;
-    double *qs = p.qstat + ((int64_t)s * p.nT + t) * 5;
-    unsigned long long *h = p.qhist + ((int64_t)s * p.nT + t) * 201;
-    const int *perm = p.perm + (int64_t)s * p.R * p.nT;
-    for (int r = 0; r < p.R; ++r) {
-        const int slot = perm[r * p.nT + t];
-        const V *x = a + sd.a_off + (int64_t)(slot - sd.chain0) * N;
-        double i2 = 0.0, i4 = 0.0, i8 = 0.0;
-        for (int k = threadIdx.x; k < N; k += blockDim.x) {
-            const V v = x[k];
-            const double u = (double)v.x * v.x + (double)v.y * v.y;
-            i2 += u; i4 += u * u; i8 += (u * u) * (u * u);
-        }
-        i2 = block_sum(i2, scratch);
-        i4 = block_sum(i4, scratch);
-        i8 = block_sum(i8, scratch);
-        if (threadIdx.x == 0) {
-            const double e = E[slot];
-            st[0] += 1.0; st[1] += e; st[2] += e * e;
-            st[3] += i4 / (i2 * i2); st[4] += i8 / (i4 * i4);
-            st[5] += i2; st[6] += i2 * i2;
-        }
-    }
-    for (int r1 = 0; r1 < p.R; ++r1)
-        for (int r2 = r1 + 1; r2 < p.R; ++r2) {
-            const V *x = a + sd.a_off + (int64_t)(perm[r1 * p.nT + t] - sd.chain0) * N;
-            const V *y = a + sd.a_off + (int64_t)(perm[r2 * p.nT + t] - sd.chain0) * N;
-            double d = 0.0;
-            for (int k = threadIdx.x; k < N; k += blockDim.x) {
-                const V u = x[k], v = y[k];
-                d += (double)u.x * v.x + (double)u.y * v.y;
-            }
-            d = block_sum(d, scratch);
-            if (threadIdx.x == 0) {
-                const double q = d / (double)N;
-                qs[0] += 1.0; qs[1] += q; qs[2] += q * q; qs[3] += q * q * q; qs[4] += (q * q) * (q * q);
-                int b = (int)floor(100.0 * (q + 1.0) + 0.5);
-                b = b < 0 ? 0 : (b > 200 ? 200 : b);
-                h[b] += 1ull;
-            }
-        }
-}
+// A task (one chain, or one pair of replicas, of one measurement) is one warp's; the sums over tasks are then taken in
+// task order, one thread per accumulator.  (One block per chain and pair in turn, with block-wide reductions: 103 us for
+// 5 measurements of 4 replicas at N = 18 on GB300, latency of the reductions.)
+constexpr int kMeasWarps = 8, kMeasBatch = 32;
 
-template <typename V> __global__ void measure_kernel(MeasureParams p) {
-    __shared__ double scratch[32];
-    const int s = blockIdx.x / p.nT, t = blockIdx.x % p.nT;
-    for (int kk = 0; kk < p.n_snap; ++kk)
-        measure_one<V>(p, reinterpret_cast<const V *>(p.snap_a) + (int64_t)kk * p.a_total,
-                       p.snap_E + (int64_t)kk * p.n_chains, s, t, scratch);
-    if (p.live) measure_one<V>(p, reinterpret_cast<const V *>(p.a), p.E, s, t, scratch);
+template <typename V> __global__ void __launch_bounds__(kMeasWarps * 32) measure_kernel(MeasureParams p) {
+    __shared__ double res[kMeasBatch][6];  // chain: E, Y2, Y4, I; pair: q
+    const int s = blockIdx.x / p.nT, t = blockIdx.x % p.nT, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const SampleDev sd = p.samples[s];
+    const int N = sd.N, R = p.R, pairs = R * (R - 1) / 2, per = R + pairs, total = (p.n_snap + (p.live ? 1 : 0)) * per;
+    const int *perm = p.perm + (int64_t)s * R * p.nT;
+    double *st = p.stat + ((int64_t)s * p.nT + t) * 7, *qs = p.qstat + ((int64_t)s * p.nT + t) * 5;
+    unsigned long long *h = p.qhist + ((int64_t)s * p.nT + t) * 201;
+    for (int b0 = 0; b0 < total; b0 += kMeasBatch) {
+        const int n = min(kMeasBatch, total - b0);
+        for (int i = warp; i < n; i += kMeasWarps) {
+            const int kk = (b0 + i) / per, task = (b0 + i) - kk * per;
+            const bool live = kk == p.n_snap;
+            const V *a = live ? reinterpret_cast<const V *>(p.a) : reinterpret_cast<const V *>(p.snap_a) + (int64_t)kk * p.a_total;
+            const double *E = live ? p.E : p.snap_E + (int64_t)kk * p.n_chains;
+            if (task < R) {
+                const int slot = perm[task * p.nT + t];
+                const V *x = a + sd.a_off + (int64_t)(slot - sd.chain0) * N;
+                double i2 = 0.0, i4 = 0.0, i8 = 0.0;
+                for (int k = lane; k < N; k += 32) {
+                    const V v = x[k];
+                    const double u = (double)v.x * v.x + (double)v.y * v.y;
+                    i2 += u; i4 += u * u; i8 += (u * u) * (u * u);
+                }
+                for (int o = 16; o; o >>= 1) {
+                    i2 += __shfl_xor_sync(0xffffffffu, i2, o);
+                    i4 += __shfl_xor_sync(0xffffffffu, i4, o);
+                    i8 += __shfl_xor_sync(0xffffffffu, i8, o);
+                }
+                if (lane == 0) { res[i][0] = E[slot]; res[i][1] = i4 / (i2 * i2); res[i][2] = i8 / (i4 * i4); res[i][3] = i2; }
+            } else {
+                int r1 = 0, left = task - R;  // the left-th pair r1 < r2
+                while (left >= R - 1 - r1) { left -= R - 1 - r1; ++r1; }
+                const int r2 = r1 + 1 + left;
+                const V *x = a + sd.a_off + (int64_t)(perm[r1 * p.nT + t] - sd.chain0) * N;
+                const V *y = a + sd.a_off + (int64_t)(perm[r2 * p.nT + t] - sd.chain0) * N;
+                double d = 0.0;
+                for (int k = lane; k < N; k += 32) {
+                    const V u = x[k], v = y[k];
+                    d += (double)u.x * v.x + (double)u.y * v.y;
+                }
+                for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                if (lane == 0) res[i][0] = d / (double)N;
+            }
+        }
+        __syncthreads();
+        const int w = threadIdx.x;
+        if (w < 7) {  // n, E, E^2, Y2, Y4, I, I^2 over the chains of the batch
+            double v = st[w];
+            for (int i = 0; i < n; ++i) {
+                if ((b0 + i) % per >= R) continue;
+                const double e = res[i][0], i2 = res[i][3];
+                v += w == 0 ? 1.0 : w == 1 ? e : w == 2 ? e * e : w == 3 ? res[i][1] : w == 4 ? res[i][2] : w == 5 ? i2 : i2 * i2;
+            }
+            st[w] = v;
+        } else if (w >= 32 && w < 38) {  // n, q, q^2, q^3, q^4 and the histogram over the pairs
+            const int m = w - 32;
+            double v = m < 5 ? qs[m] : 0.0;
+            for (int i = 0; i < n; ++i) {
+                if ((b0 + i) % per < R) continue;
+                const double q = res[i][0];
+                if (m < 5) v += m == 0 ? 1.0 : m == 1 ? q : m == 2 ? q * q : m == 3 ? q * q * q : (q * q) * (q * q);
+                else {
+                    int b = (int)floor(100.0 * (q + 1.0) + 0.5);
+                    b = b < 0 ? 0 : (b > 200 ? 200 : b);
+                    h[b] += 1ull;
+                }
+            }
+            if (m < 5) qs[m] = v;
+        }
+        __syncthreads();
+    }
 }
 
 cudaError_t launch_measure(const MeasureParams &p, cudaStream_t s) {
     if (p.n_snap <= 0 && !p.live) return cudaSuccess;
-    if (p.dbl) measure_kernel<double2><<<p.S * p.nT, 128, 0, s>>>(p);
-    else measure_kernel<float2><<<p.S * p.nT, 128, 0, s>>>(p);
+    if (p.dbl) measure_kernel<double2><<<p.S * p.nT, kMeasWarps * 32, 0, s>>>(p);
+    else measure_kernel<float2><<<p.S * p.nT, kMeasWarps * 32, 0, s>>>(p);
     return cudaGetLastError();
 }
 
