@@ -563,7 +563,8 @@ template <int G, int NCW, int C> cudaError_t launch_comb_t(const SweepParams &p,
     if (q.nst == 0) return cudaErrorInvalidConfiguration;
     const size_t sm = comb_smem<G, NCW, C>(p.maxN, q.nst).total;
     auto *k = comb_sweep_kernel<G, NCW, C>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // the kernel's largest limit, not this context's: contexts of other sizes launch it too
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit());
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(clusters * C);
@@ -586,7 +587,7 @@ template <int G, int NCW, int C> int comb_clusters_t(int maxN, int sms) {
     const size_t sm = comb_smem<G, NCW, C>(maxN, d).total;
     auto *k = comb_sweep_kernel<G, NCW, C>;
     int nb = 0;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit());
     if (e == cudaSuccess && C == 1) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, (NCW + 1) * 32, sm);
         nb *= sms;

@@ -900,19 +900,23 @@ size_t variant_smem(int var, const GraphParams &p) {
 }
 }  // namespace
 
+// The limits are the kernels' largest, not this context's: they belong to the kernel, and contexts of other sizes launch it too.
 cudaError_t graph_prepare(const GraphParams &p) {
-    const int var = graph_variant(p), sm = (int)variant_smem(var, p);
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int most = (int)kGraphSmemMax, mode = 2048 * (int)sizeof(float2);
     cudaError_t e = cudaSuccess;
     TabShape t;
-    if (var == kWarp) e = cudaFuncSetAttribute(graph_warp_kernel, at, sm);
-    else if (var == kTable && table_shape(p, &t)) {
-        e = t.GC == 8 ? cudaFuncSetAttribute(graph_table_kernel<8, kTabThreads>, at, sm)
-                      : cudaFuncSetAttribute(graph_table_kernel<4, kTabThreads>, at, sm);
-    } else if (var == kStage) e = cudaFuncSetAttribute(graph_sweep_kernel<kStage>, at, sm);
-    else e = cudaFuncSetAttribute(graph_sweep_kernel<kPlain>, at, sm);
-    const int se = p.maxN * kGRS * (int)sizeof(float2);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(graph_energy_kernel, at, se);
+    switch (graph_variant(p)) {
+        case kWarp: e = cudaFuncSetAttribute(graph_warp_kernel, at, mode); break;
+        case kTable:
+            table_shape(p, &t);
+            e = t.GC == 8 ? cudaFuncSetAttribute(graph_table_kernel<8, kTabThreads>, at, most)
+                          : cudaFuncSetAttribute(graph_table_kernel<4, kTabThreads>, at, most);
+            break;
+        case kStage: e = cudaFuncSetAttribute(graph_sweep_kernel<kStage>, at, most); break;
+        default: e = cudaFuncSetAttribute(graph_sweep_kernel<kPlain>, at, most);
+    }
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(graph_energy_kernel, at, kGRS * mode);
     return e;
 }
 

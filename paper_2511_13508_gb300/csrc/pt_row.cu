@@ -21,6 +21,7 @@ namespace ptgb {
 
 namespace {
 
+constexpr int kRowSmemMax = 227 * 1024;
 constexpr int kRowDraws = 32;  // updates whose random numbers are drawn at once, one lane each
 
 // Pair products in rows by p, the pair's distance from the middle of its sum: pair {x, s-x}, x < s-x, is the p-th of
@@ -336,10 +337,11 @@ size_t row_smem_bytes(bool dbl, int maxN) { return dbl ? RowSmem<double>(maxN).t
     else if (maxN <= 64) { auto *k = row_sweep_kernel<T, 0, 160, kF ? 5 : 6>; CALL; }                 \
     else { auto *k = row_sweep_kernel<T, 0, kRowMaxThreads, 1>; CALL; }
 
+// The limit is the kernel's largest (kRowSmemMax), not this context's: contexts of other sizes launch the same kernel.
 cudaError_t row_prepare(bool dbl, int maxN) {
-    const int sm = (int)row_smem_bytes(dbl, maxN);
-    if (dbl) { PT_ROW_DISPATCH(double, return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)) }
-    else { PT_ROW_DISPATCH(float, return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)) }
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (dbl) { PT_ROW_DISPATCH(double, return cudaFuncSetAttribute(k, at, kRowSmemMax)) }
+    else { PT_ROW_DISPATCH(float, return cudaFuncSetAttribute(k, at, kRowSmemMax)) }
 }
 
 cudaError_t launch_row_sweep(bool dbl, const RowParams &p, cudaStream_t s) {

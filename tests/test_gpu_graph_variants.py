@@ -66,3 +66,21 @@ def test_graph_without_quadruplets():
     p.sweep(4)
     o = p.observables()
     assert np.array_equal(o["mc_acc"], o["mc_att"]) and np.all(p.state()[1] == 0.0)
+
+
+@pytest.mark.parametrize("make", ["random", "sparse", "row", "comb"])
+def test_contexts_of_other_sizes_keep_running(make):
+    """A kernel's shared-memory limit serves every context that launches it: a larger context sweeps (with a new launch
+    shape) after smaller ones were made."""
+    def one(N):
+        temps = workload.geometric_ladder(0.3, 1.6, 4)
+        if make in ("random", "sparse"):
+            graphs, Js = random_graphs([N]) if make == "random" else sparse_graphs([8 * N], 4)
+            return pkg.PT([N if make == "random" else 8 * N], Js, temps, 1, 3, precision="fp32", graphs=graphs)
+        Js = [workload.couplings(N, len(pkg.enumerate_quads(N)), 4)]
+        kw = dict(precision="fp64") if make == "row" else dict(precision="fp32", chains_per_block=8)
+        return pkg.PT([N], Js, temps, 1, 3, **kw)
+    a, b = one(64), one(40)
+    b.sweep(1)
+    a.sweep(2)
+    assert np.isfinite(a.state()[1]).all() and np.isfinite(b.state()[1]).all() and np.isfinite(a.energy()).all()
