@@ -536,9 +536,9 @@ int learn_backward(pt_ctx *c, int rows, const int *cond) {
     w1.A = L.dZ1T; w1.strideA = rc * sh.H; w1.B = L.XT; w1.strideB = rc * sh.Din;
     w1.M = sh.H; w1.N = sh.Din; w1.D = L.Gr + sh.oW1; w1.ldd = sh.Din;
     CK(launch_gemm_bf16(w1, c->S, c->stream));
-    CK(launch_colsum(L.dO, rows, sh.Dout, L.Gr + sh.ob3, nullptr, nullptr, c->S, rc * sh.Dout, ps, c->stream));
-    CK(launch_colsum(L.dZ2, rows, sh.H, L.Gr + sh.ob2, nullptr, nullptr, c->S, rc * sh.H, ps, c->stream));
-    CK(launch_colsum(L.dZ1, rows, sh.H, L.Gr + sh.ob1, L.Gr + sh.oC1, cond, c->S, rc * sh.H, ps, c->stream));
+    CK(launch_colsum(L.dO, rows, sh.Dout, L.Gr + sh.ob3, nullptr, nullptr, 0, c->S, rc * sh.Dout, ps, c->stream));
+    CK(launch_colsum(L.dZ2, rows, sh.H, L.Gr + sh.ob2, nullptr, nullptr, 0, c->S, rc * sh.H, ps, c->stream));
+    CK(launch_colsum(L.dZ1, rows, sh.H, L.Gr + sh.ob1, L.Gr + sh.oC1, cond, sh.ncold, c->S, rc * sh.H, ps, c->stream));
     return PT_OK;
 }
 
@@ -790,11 +790,12 @@ void incidence_records(int N, const int32_t *abcd, const double *J, const int *o
         }
 }
 
-// f(s) for every sample, over the host's cores.  False when a call ran out of memory.
-template <typename F> bool for_samples(int S, F &&f) {
+// f(s) for every sample, over the host's cores when there is `work` (entries in all) enough to start threads for.  False
+// when a call ran out of memory.
+template <typename F> bool for_samples(int S, int64_t work, F &&f) {
     std::atomic<int> next{0};
     std::atomic<bool> ok{true};
-    auto work = [&]() {
+    auto run = [&]() {
         try {
             for (int s = next++; s < S; s = next++) f(s);
         } catch (const std::bad_alloc &) {
@@ -802,13 +803,13 @@ template <typename F> bool for_samples(int S, F &&f) {
         }
     };
     std::vector<std::thread> pool;
-    const int n = std::min({S, 16, std::max(1, (int)std::thread::hardware_concurrency())});
+    const int n = work < (1 << 16) ? 1 : std::min({S, 16, std::max(1, (int)std::thread::hardware_concurrency())});
     try {
         pool.reserve(n);
-        for (int i = 1; i < n; ++i) pool.emplace_back(work);
+        for (int i = 1; i < n; ++i) pool.emplace_back(run);
     } catch (const std::exception &) {  // no more threads: the ones there are, and this one, do the work
     }
-    work();
+    run();
     for (auto &t : pool) t.join();
     return ok;
 }
@@ -1293,7 +1294,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
                 incidence_records(n, abcd.data(), J + J_offsets[s], offs[s].data(), hinc.data() + sd.inc_off,
                                   hrec.data() + sd.inc_off, hrecJ.data() + sd.inc_off);
         };
-        if (!for_samples(S, build)) return bail(fail(c, PT_ENOMEM, "host allocation failed (quadruplet lists)"));
+        if (!for_samples(S, q_off, build)) return bail(fail(c, PT_ENOMEM, "host allocation failed (quadruplet lists)"));
         for (int s = 0; s < S; ++s) {
             for (int l = 0; l < c->N[s]; ++l) c->max_deg = std::max(c->max_deg, offs[s][l + 1] - offs[s][l]);
             hinc_off.insert(hinc_off.end(), offs[s].begin(), offs[s].end());
@@ -1305,7 +1306,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
                 graph_lists(c->N[s], sd.nq, graph + 4 * J_offsets[s], J + J_offsets[s], offs[s].data(), hrec.data() + sd.inc_off,
                             hrecJ.data() + sd.inc_off, lists[s]);
             };
-            if (!for_samples(S, make)) return bail(fail(c, PT_ENOMEM, "host allocation failed (graph lists)"));
+            if (!for_samples(S, 10 * q_off, make)) return bail(fail(c, PT_ENOMEM, "host allocation failed (graph lists)"));
             int64_t nch = 0, ncr = 0, nco = 0, nxo = 0;
             for (int s = 0; s < S; ++s) {
                 SampleDev &sd = c->samples[s];

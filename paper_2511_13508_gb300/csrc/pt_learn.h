@@ -81,7 +81,7 @@ struct DensityParams {
 cudaError_t launch_density(const DensityParams &p, int S, cudaStream_t s);
 
 // Bias gradients: db[col] = sum_rows dZ[row][col]; dC[cond[row]][col] += dZ[row][col] (optional)
-cudaError_t launch_colsum(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond, int S,
+cudaError_t launch_colsum(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond, int ncond, int S,
                           int64_t strideZ, int64_t strideGrad, cudaStream_t s);
 
 // Adam on [S][psize] parameters (grad G already averaged).
