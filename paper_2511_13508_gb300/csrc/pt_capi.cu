@@ -55,6 +55,7 @@ struct SampleLayout {
     int N, ST, nblk;
     std::vector<int> bo, xtlo, mode_blk, ebo;
     std::vector<uint32_t> blkinfo;
+    std::vector<int> eseg;  // prefix over the blocks of their runs of kEnergySeg modes l that use the block in H
     int64_t jblocks;  // blocks of J stored for the sample
 };
 
@@ -92,6 +93,12 @@ SampleLayout make_layout(int N) {
         L.ebo[l + 1] = L.ebo[l] + (sta <= sthi ? L.bo[sthi + 1] - L.bo[sta] : 0);
     }
     L.jblocks = L.mode_blk[N];
+    L.eseg.assign(L.nblk + 1, 0);
+    for (int b = 0; b < L.nblk; ++b) {
+        const int s0 = (int)(L.blkinfo[b] >> 16) * TS, x0 = (int)(L.blkinfo[b] & 0xffffu) * TX;
+        const int lo = std::max(0, s0 - N + 1), hi = std::min(x0 + TX - 1, N);  // modes [lo, hi)
+        L.eseg[b + 1] = L.eseg[b] + (hi > lo ? (hi - lo + kEnergySeg - 1) / kEnergySeg : 0);
+    }
     return L;
 }
 
@@ -197,7 +204,7 @@ struct pt_ctx {
     SampleDev *d_samples = nullptr;
     GroupDev *d_groups = nullptr;
     void *d_J = nullptr;
-    int *d_bo = nullptr, *d_xtlo = nullptr, *d_mode_blk = nullptr, *d_ebo = nullptr;
+    int *d_bo = nullptr, *d_xtlo = nullptr, *d_mode_blk = nullptr, *d_ebo = nullptr, *d_eseg = nullptr;
     uint32_t *d_blkinfo = nullptr;
     void *d_a = nullptr;
     double *d_E = nullptr, *d_beta = nullptr, *d_Etmp = nullptr;
@@ -357,12 +364,19 @@ int run_energy(pt_ctx *c, int renorm, double *E_out, bool write_state) {
     p.samples = c->d_samples; p.groups = c->d_groups; p.J = c->d_J; p.bo = c->d_bo; p.blkinfo = c->d_blkinfo;
     p.mode_blk = c->d_mode_blk; p.ebo = c->d_ebo; p.a = c->d_a; p.cc = c->cfg.cc_factor; p.renorm = renorm;
     p.E_out = E_out; p.E_state = write_state ? c->d_E : nullptr; p.ctl = c->d_ctl;
-    // several thread blocks per group (their partial sums added in a fixed order by a second kernel), so that the
-    // resync fills the GPU with more warps than one block per group gives (about 8 blocks per SM; measured on
-    // GB300: see the energy kernel)
-    const int ng = (int)c->groups.size();
-    p.part = c->d_epart;
-    p.parts = std::max(1, std::min(kEnergyPartsMax, (8 * std::max(c->sms, 1) + ng - 1) / std::max(ng, 1)));
+    // several thread blocks per group, their partial sums added in a fixed order by a second kernel.  FP64: about 8 blocks
+    // per SM (it waits on coupling loads).  FP32: one block per SM at a time, so the number of parts that leaves the least
+    // of the last wave idle, each part counted with the 2% that loading the group's tables takes
+    const int ng = (int)c->groups.size(), sms = std::max(c->sms, 1);
+    p.part = c->d_epart; p.eseg = c->d_eseg; p.maxN = c->maxN;
+    if (c->dbl) p.parts = std::max(1, std::min(8, (8 * sms + ng - 1) / std::max(ng, 1)));
+    else {
+        double best = 1e30;
+        for (int q = 1; q <= kEnergyPartsMax; ++q) {
+            const double t = (double)((ng * q + sms - 1) / sms) / q * (1.0 + 0.02 * q);
+            if (t < best) { best = t; p.parts = q; }
+        }
+    }
     const int Ge = c->dbl ? std::min(c->G, 16) : c->G;
     CK(launch_energy(c->dbl, Ge, p, ng, c->maxN, c->stream));
     return PT_OK;
@@ -1180,7 +1194,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
 
     // ---- samples, chains, groups, layouts
     std::vector<SampleLayout> lay(S);
-    std::vector<int> bo_all, xtlo_all, mode_all, ebo_all;
+    std::vector<int> bo_all, xtlo_all, mode_all, ebo_all, eseg_all;
     std::vector<uint32_t> binfo_all;
     if (!c->plain && !c->gfp32 && cfg.chains_per_block == 0 && cfg.consumer_warps == 0)
         c->row = row_path(c->dbl, c->maxN, (int64_t)S * chains_ps, sms);
@@ -1194,6 +1208,8 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         sd.J_off = jblocks; sd.a_off = a_off; sd.q_off = q_off; sd.nq = J_offsets[s + 1] - J_offsets[s];
         sd.inc_off = inc_total;
         sd.row_off = row_total;
+        sd.seg_off = (int)eseg_all.size();
+        eseg_all.insert(eseg_all.end(), lay[s].eseg.begin(), lay[s].eseg.end());
         bo_all.insert(bo_all.end(), lay[s].bo.begin(), lay[s].bo.end());
         xtlo_all.insert(xtlo_all.end(), lay[s].xtlo.begin(), lay[s].xtlo.end());
         xtlo_all.push_back(0);
@@ -1228,6 +1244,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     RC(dalloc(c, &c->d_blkinfo, std::max<size_t>(1, binfo_all.size())));
     RC(dalloc(c, &c->d_mode_blk, mode_all.size()));
     RC(dalloc(c, &c->d_ebo, ebo_all.size()));
+    RC(dalloc(c, &c->d_eseg, eseg_all.size()));
     c->d_a = dev_alloc(c, (size_t)c->a_total * 2 * c->esize);
     if (!c->d_a) return bail(fail(c, PT_ENOMEM, "device allocation failed (state)"));
     c->d_snap_a = dev_alloc(c, (size_t)c->n_snap_max * c->a_total * 2 * c->esize);
@@ -1363,6 +1380,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     if (!binfo_all.empty()) CK(cudaMemcpy(c->d_blkinfo, binfo_all.data(), binfo_all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_mode_blk, mode_all.data(), mode_all.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_ebo, ebo_all.data(), ebo_all.size() * sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(c->d_eseg, eseg_all.data(), eseg_all.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_label, label.data(), label.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_perm, perm.data(), perm.size() * sizeof(int), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->d_chain_sample, c->chain_sample.data(), c->chain_sample.size() * sizeof(int), cudaMemcpyHostToDevice));

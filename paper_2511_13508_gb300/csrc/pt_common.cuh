@@ -94,6 +94,7 @@ struct SampleDev {
     int64_t q_off;   // offset of the sample in the canonical quadruplet arrays (plain path)
     int64_t nq;      // quadruplets of the sample
     int64_t inc_off; // offset of the sample in the incidence arrays (plain path), N+1 entries at mode_off
+    int seg_off;     // offset of the sample in the energy kernel's tile prefix (nblk+1 entries)
     int64_t chunk_off, cross_off, xoff_off;  // pair-table graph sweep: chunks, cross entries, pair offsets of the sample
     int64_t row_off; // offset of the sample in the row store (row path), N * N/2 * N entries
 };

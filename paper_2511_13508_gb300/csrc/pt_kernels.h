@@ -68,8 +68,13 @@ struct EnergyParams {
     Control *ctl;
     double *part;    // partial sums [group][part][32] (kEnergyPartsMax parts at most)
     int parts;       // thread blocks per group (1 .. kEnergyPartsMax)
+    const int *eseg; // FP32, per sample: prefix count over the tiles (blocks) of their runs of modes (nblk+1, at seg_off)
+    int maxN;
 };
-constexpr int kEnergyPartsMax = 8;
+constexpr int kEnergyPartsMax = 16;
+constexpr int kEnergySeg = 64;  // modes of a run
+// pt_energy.cu: the partial sums of FP32 chains
+cudaError_t launch_energy_tiles(int G, const EnergyParams &p, int ngroups, cudaStream_t s);
 
 // pt_comb.cu: FP32 comb sweep, G chains per group (on a cluster of cl blocks), ncw field warps per block
 bool comb_variant_exists(int G, int ncw, int cl);

@@ -730,14 +730,10 @@ __global__ void fields_kernel(FieldsParams prm) {
 // keeps only the pairs {p, q} of row x+m whose smaller mode (the block column) exceeds x,
 //     H = -cc sum_x Re( conj(a_x) h^>_x ),
 // which visits every quadruplet once, at its smallest mode x (partner m: the largest; the pair {p, q} of
-// the two middle modes has p > x).  Blocks whose columns all lie at or below x are skipped.  Products and
-// row sums in `real`, per-block sums accumulated in FP64.  A group's blocks are split over prm.parts thread
-// blocks (block b of part p takes the work items p NW + worker, stepping by parts NW); each writes its per-chain
-// FP64 sums to prm.part and energy_sum_kernel adds the parts in order.  With renorm != 0, renorm_kernel first
-// rescales every chain onto sum |a|^4 = N.  The kernel waits on coupling loads from L2, so it runs as many
-// warps per SM as fit: 3 blocks of 256 threads (FP32; 2 for FP64) and about 8 blocks per SM in all.  Measured on
-// GB300 (resync of the N = 256 bench workload, 192 groups): 2.81 ms with one block per group, 2.08 ms with about
-// 4 blocks per SM at 2 per SM, 1.45 ms now; batched N = 64: 0.166 -> 0.12 ms, ragged batch: 0.58 -> 0.24 ms.
+// the two middle modes has p > x).  A group's share is split over prm.parts thread blocks, each writing per-chain FP64
+// sums to prm.part, and energy_sum_kernel adds the parts in order.  With renorm != 0, renorm_kernel first rescales every
+// chain onto sum |a|^4 = N.  FP32 chains: energy_tile_kernel (pt_energy.cu).  FP64: energy_kernel, whose work items are
+// (mode, block); it waits on coupling loads from L2, so it runs about 8 blocks per SM in all.
 template <typename real, int G>
 __global__ void __launch_bounds__(256) renorm_kernel(EnergyParams prm) {
     using V = typename vec2<real>::type;
@@ -766,7 +762,7 @@ __global__ void __launch_bounds__(256) renorm_kernel(EnergyParams prm) {
 }
 
 template <typename real, int G>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2) energy_kernel(EnergyParams prm) {
+__global__ void __launch_bounds__(256, 2) energy_kernel(EnergyParams prm) {
     using V = typename vec2<real>::type;
     constexpr int RS = RowStride<real, G>::value, NCW = 8, WPW = 32 / G, NW = NCW * WPW;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -942,15 +938,20 @@ template <typename real, int G>
 static cudaError_t launch_energy_t(const EnergyParams &p, int ngroups, int maxN, cudaStream_t s) {
     using V = typename vec2<real>::type;
     const size_t sm = (size_t)(maxN + 2 * APAD) * RowStride<real, G>::value * sizeof(V) + 8 * G * sizeof(double) + 64;
-    cudaError_t e = cudaFuncSetAttribute(energy_kernel<real, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(real) == 8) e = cudaFuncSetAttribute(energy_kernel<real, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     if (p.parts < 1 || p.parts > kEnergyPartsMax || !p.part) return cudaErrorInvalidValue;
     if (p.renorm) {
         renorm_kernel<real, G><<<ngroups, 256, 0, s>>>(p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    energy_kernel<real, G><<<ngroups * p.parts, 256, sm, s>>>(p);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if constexpr (sizeof(real) == 4) e = launch_energy_tiles(G, p, ngroups, s);
+    else {
+        energy_kernel<real, G><<<ngroups * p.parts, 256, sm, s>>>(p);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
     energy_sum_kernel<<<ngroups, 32, 0, s>>>(p);
     return cudaGetLastError();
 }
