@@ -187,6 +187,7 @@ struct pt_ctx {
     void *d_Jrow = nullptr;  // its coupling store (null: the context does not take that path)
     int *d_order = nullptr;  // chain slots, largest N first
     int cl = 1;              // thread blocks per group (FP32 comb sweep)
+    int most = 1;            // groups the device sweeps at once
     cudaStream_t stream = nullptr;
     pt_alloc_fn alloc = nullptr;
     pt_free_fn free_ = nullptr;
@@ -319,6 +320,21 @@ bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
     return maxN <= 48 && n_chains <= (maxN <= 32 ? 6 : 2) * (int64_t)sms;
 }
 
+// Runs each group's updates are cut into on a device that holds `most` groups at once: those that leave the least of the last
+// round of units idle.  A unit costs about 8 us beside its updates (tables, amplitudes, the first couplings), an update of
+// the largest N about 2 + N^2 / 6000 us (GB300).
+int sweep_runs(int groups, int most, int64_t updates, int maxN) {
+    const double group_us = (double)updates * (2.0 + maxN * (double)maxN / 6000.0);
+    const int top = (int)std::max<int64_t>(1, std::min<int64_t>(updates, 512));
+    int best = 1;
+    double best_t = 1e300;
+    for (int k = 1; k <= top; ++k) {
+        const double t = (double)(((int64_t)groups * k + most - 1) / std::max(most, 1)) * (group_us / k + 8.0);
+        if (t < best_t) { best_t = t; best = k; }
+    }
+    return best;
+}
+
 // Blocks per group of the FP32 sweep (a cluster) when its groups leave SMs idle: the most that keep all groups resident
 // at once, and no more than an update has chunks for.  Measured on GB300 (us per sweep of one sample, 8 chains x 7
 // warps, 1 / 2 / 4 / 8 blocks): N = 256, 12 groups 1680 / 1057 / 633 / 428; N = 160, 8 groups 509 / 349 / 247 / 180;
@@ -442,8 +458,9 @@ int run_sweeps(pt_ctx *c, int seg) {
     p.progress = c->d_progress; p.n_sweeps = seg; p.sweeps_per_unit = std::min(c->spu, seg);
     p.measure_every = c->cfg.measure_every; p.snap_a = c->d_snap_a; p.snap_E = c->d_snap_E;
     p.n_snap_max = c->n_snap_max; p.a_total = c->a_total; p.n_chains = c->n_chains; p.trace = c->d_trace;
-    const int units = ((seg + p.sweeps_per_unit - 1) / p.sweeps_per_unit) * p.n_groups;
-    const int grid = std::max(1, std::min(c->grid, units));
+    p.runs = (seg + p.sweeps_per_unit - 1) / p.sweeps_per_unit;
+    if (!c->dbl && c->cfg.sweeps_per_unit == 0) p.runs = sweep_runs(p.n_groups, c->most, (int64_t)seg * (c->maxN / 2), c->maxN);
+    const int grid = std::max(1, std::min(c->grid, p.runs * p.n_groups));
     if (!c->dbl) CK(launch_comb(c->G, c->ncw, c->cl, p, grid, c->stream));
     else CK(launch_sweep(c->dbl, c->G, c->ncw, p, grid, c->stream));
     return PT_OK;
@@ -752,6 +769,7 @@ int set_shape(pt_ctx *c, int G, int ncw, int spu) {
     }
     CK(cudaMemcpy(c->d_groups, c->groups.data(), c->groups.size() * sizeof(GroupDev), cudaMemcpyHostToDevice));
     if (c->cfg.blocks_per_sm > 0) most = std::min(most, sms * c->cfg.blocks_per_sm);
+    c->most = most;
     c->grid = std::max(1, std::min((int)c->groups.size(), most));
     c->G = G; c->ncw = ncw; c->spu = spu;
     c->row = false;
@@ -1411,6 +1429,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         int most = shape_groups(c, G, ncw, c->cl, sms);
         if (most < 1) return bail(fail(c, PT_EUNSUPPORTED, "pt_create: sweep kernel does not fit on this GPU for this N"));
         if (cfg.blocks_per_sm > 0) most = std::min(most, sms * cfg.blocks_per_sm);
+        c->most = most;
         c->grid = std::max(1, std::min((int)c->groups.size(), most));
         c->sms = sms;
         RC(dalloc(c, &c->d_epart, c->max_groups * (size_t)kEnergyPartsMax * 32));

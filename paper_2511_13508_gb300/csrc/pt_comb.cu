@@ -212,7 +212,8 @@ template <int G, int NCW, int C> __host__ __device__ CombSmem comb_smem(int maxN
 // NCW field warps and a copy warp.  A lane is (chain c = lane % G, worker lane / G of its warp); worker w takes block w of
 // every chunk of CB blocks.  The copy warp streams the J runs of j and k into a ring of nst stages and fills one slot
 // per update with the B_jk couplings and the random part of every chain's proposal.  Work units (group, run of sweeps)
-// come from a ticket counter; a unit waits (bounded) until the previous run of its group has been written back.
+// come from a ticket counter; a unit waits (bounded) until the previous run of its group has been written back.  A run need
+// not end with a sweep: the launcher cuts each group's updates into as many equal runs as balance the SMs best.
 template <int G, int NCW, int C>
 __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepParams p) {
     using Sh = CombShape<G, NCW>;
@@ -252,8 +253,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
     };
 
     const long long sweep_base = p.ctl->sweep_base;
-    const int n_sweeps = p.n_sweeps, spu = p.sweeps_per_unit;
-    const unsigned units = (unsigned)((n_sweeps + spu - 1) / spu) * (unsigned)p.n_groups;
+    const int n_sweeps = p.n_sweeps;
+    const unsigned units = (unsigned)p.runs * (unsigned)p.n_groups;
     const float *J = reinterpret_cast<const float *>(p.J);
     float2 *A = reinterpret_cast<float2 *>(p.a);
     uint32_t q = 0;  // chunks so far (ring position); stage and phase advance with it, without a division
@@ -294,7 +295,8 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
         const GroupDev gr = p.groups[g];
         const SampleDev sd = p.samples[gr.sample];
         const int N = sd.N, half = N / 2;
-        const int sw0 = ci * spu, sw1 = min(n_sweeps, sw0 + spu);
+        // updates [n0, n1) of the group's n_sweeps * half
+        const int n0 = (int)((long long)n_sweeps * half * ci / p.runs), n1 = (int)((long long)n_sweeps * half * (ci + 1) / p.runs);
         const int *mode_blk = p.mode_blk + sd.mode_off;
         // identity of chain c (the Philox stream of its proposals): (sample, replica, temperature its slot holds)
         uint32_t id = 0u;
@@ -307,12 +309,11 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
 
         if (producer) {
             const int *bo_g = p.bo + sd.tab_off, *xtlo_g = p.xtlo + sd.tab_off;
-            bool stop = false;
-            for (int sw = sw0; sw < sw1 && !stop; ++sw) {
-                const uint32_t sweep = (uint32_t)(sweep_base + sw);
-                for (int u = 0; u < half; ++u) {
-                    stop = __shfl_sync(0xffffffffu, *abort_flag, 0) != 0;  // warp-uniform
-                    if (stop) break;
+            int sw = n0 / half, u = n0 - sw * half;
+            {
+                for (int n = n0; n < n1; ++n, u = u + 1 == half ? (++sw, 0) : u + 1) {
+                    const uint32_t sweep = (uint32_t)(sweep_base + sw);
+                    if (__shfl_sync(0xffffffffu, *abort_flag, 0) != 0) break;  // warp-uniform
                     int j, k;
                     pair_jk(p.seed, (uint32_t)gr.sample, sweep, (uint32_t)u, N, j, k);
                     const Ranges Rg = update_ranges(sd, bo_g, mode_blk, j, k);
@@ -370,8 +371,10 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
         const int tr_u = p.trace ? p.ctl->trace_update : -1;
         const float cc = (float)p.cc;
 
-        for (int sw = sw0; sw < sw1; ++sw) {
+        for (int n = n0; n < n1;) {
+            const int sw = n / half, u0 = n - sw * half, u1 = min(half, u0 + n1 - n);
             const uint32_t sweep = (uint32_t)(sweep_base + sw);
+            n += u1 - u0;
             // the sweep's pair sequence (every warp has read the previous sweep's last entry before that update's barrier)
             for (int i = tid; i < half; i += NCT) {
                 int j, k;
@@ -379,7 +382,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
                 s_pair[i] = j | (k << 16);
             }
             named_bar(1, NCT);
-            for (int u = 0; u < half; ++u, ++upd) {
+            for (int u = u0; u < u1; ++u, ++upd) {
                 const int jk = s_pair[u], j = jk & 0xffff, k = jk >> 16;
                 const Ranges Rg = update_ranges(sd, s_bo, mode_blk, j, k);
                 const int buf = (int)(upd & 1u);
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
             }
             // interior measurement point: snapshot amplitudes and energies
             const long long done = sweep_base + sw + 1;
-            if (p.measure_every > 0 && done % p.measure_every == 0 && sw + 1 < n_sweeps) {
+            if (u1 == half && p.measure_every > 0 && done % p.measure_every == 0 && sw + 1 < n_sweeps) {
                 const int kk = (int)(done / p.measure_every - sweep_base / p.measure_every - 1);
                 named_bar(1, NCT);
                 if (rank == 0 && kk >= 0 && kk < p.n_snap_max) {
@@ -520,7 +523,7 @@ __global__ void __launch_bounds__((NCW + 1) * 32, 1) comb_sweep_kernel(SweepPara
                 const int slot = gr.chain0 + tid;
                 __stcg(p.E + slot, E);
                 p.mc_acc[slot] += n_acc;
-                p.mc_att[slot] += (unsigned long long)(sw1 - sw0) * half;
+                p.mc_att[slot] += (unsigned long long)(n1 - n0);
             }
             __threadfence();
             named_bar(1, NCT);

@@ -37,6 +37,7 @@ struct SweepParams {
     // pre-update states [a_total] as double complex, both in canonical (sample, replica, temperature) order
     double *trace;
     int nst;                    // coupling ring stages (set by the launcher)
+    int runs;                   // FP32 comb sweep: runs of updates a group's work is cut into
 };
 
 struct FieldsParams {
