@@ -46,6 +46,13 @@ template <typename V> __device__ __forceinline__ V pair_product(V lo, V hi) {
     return r;
 }
 
+// A proposal as the rows use it.  test: FP32 the Metropolis uniform U; FP64 log U / (beta cc), drawn once with the proposal,
+// so that the decision is one comparison: dH = -cc share, and U < exp(-beta dH) is share > log U / (beta cc), which holds for
+// every dH <= 0 because log U < 0.
+template <typename real> struct RowProposal {
+    typename vec2<real>::type aj, ak, nj, nk, dj, dk;
+    real test;
+};
 template <typename real> struct RowSmem {
     size_t a, draws, prop, part, pairs, total;
     __host__ __device__ RowSmem(int N) {
@@ -55,16 +62,15 @@ template <typename real> struct RowSmem {
         draws = a + (size_t)N * sizeof(V);
         draws = (draws + 15) / 16 * 16;
         prop = draws + 2 * kRowDraws * sizeof(ProposalDraw<real>);
-        part = prop + 4 * sizeof(Proposal<real>);
+        part = prop + 4 * sizeof(RowProposal<real>);
         pairs = part + 2 * 32 * sizeof(real);
         total = pairs + 2 * kRowDraws * sizeof(int);
     }
 };
 
-// FP64: the acceptance test on log U, drawn once with the proposal instead of an exponential per update.
-template <typename real> __device__ __forceinline__ bool row_accept(real dH, real beta, real U) {
-    if constexpr (sizeof(real) == 4) return metropolis_accept(dH, beta, U);
-    else return dH <= real(0) || U < -beta * dH;
+template <typename real> __device__ __forceinline__ bool row_accept(real share, real dH, real beta, real test) {
+    if constexpr (sizeof(real) == 4) return metropolis_accept(dH, beta, test);
+    else return share > test;
 }
 
 }  // namespace
@@ -85,7 +91,7 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
     V *z = reinterpret_cast<V *>(smem);
     V *a = reinterpret_cast<V *>(smem + lay.a);
     ProposalDraw<real> *draws = reinterpret_cast<ProposalDraw<real> *>(smem + lay.draws);  // [2][kRowDraws]
-    Proposal<real> *prop = reinterpret_cast<Proposal<real> *>(smem + lay.prop);            // [2][2]
+    RowProposal<real> *prop = reinterpret_cast<RowProposal<real> *>(smem + lay.prop);      // [2][2]
     real *part = reinterpret_cast<real *>(smem + lay.part);                                // [2][32]
     int *pairs = reinterpret_cast<int *>(smem + lay.pairs);                                // [2][kRowDraws]
 
@@ -114,7 +120,7 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
             pair_jk(p.seed, (uint32_t)si, (uint32_t)(base + sw), (uint32_t)u, N, j, k);
             pairs[at] = j | (k << 16);
             ProposalDraw<real> D = draw_proposal<real>(p.seed, cid, (uint32_t)(base + sw), (uint32_t)u);
-            if constexpr (sizeof(real) == 8) { D.pad = D.U; D.U = log(D.U); }
+            if constexpr (sizeof(real) == 8) { D.pad = D.U; D.U = log(D.U) / (beta * cc); }
             draws[at] = D;
         }
     };
@@ -147,16 +153,22 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
         }
     };
     if (has_row && total > 0) row_of(pairs[0]);
+    auto propose = [&](RowProposal<real> &o, const ProposalDraw<real> &D, V aj, V ak) {
+        const Proposal<real> P = finish_proposal<real>(D, aj, ak);
+        o.aj = aj; o.ak = ak; o.nj = P.nj; o.nk = P.nk; o.test = P.U;
+        o.dj.x = P.nj.x - aj.x; o.dj.y = P.nj.y - aj.y;
+        o.dk.x = P.nk.x - ak.x; o.dk.y = P.nk.y - ak.y;
+    };
     if (helper && lane < 2 && total > 0) {
         const int jk = pairs[0];
-        prop[lane] = finish_proposal<real>(draws[0], a[jk & 0xffff], a[jk >> 16]);
+        propose(prop[lane], draws[0], a[jk & 0xffff], a[jk >> 16]);
     }
     __syncthreads();
 
     int ok = 0, at_u = 0, sw = 0;
     for (int i = 0; i < total; ++i) {
         const int jk = pairs[i & (2 * kRowDraws - 1)], j = jk & 0xffff, k = jk >> 16;
-        const Proposal<real> &P = prop[(i & 1) * 2 + ok];
+        const RowProposal<real> &P = prop[(i & 1) * 2 + ok];
         const bool traced = tr_at == base + sw + 1 && at_u == tr_u;
         real share = 0;
         V acc;
@@ -166,9 +178,10 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
             ac2.x = ac2.y = real(0);
             int zi = s - 1, step = 2 * N - 5;
             if constexpr (NP > 0) {
+                // past the row's end the coupling is zero and the product any one: no branches
 #pragma unroll
                 for (int e = 0; e < NP; ++e) {
-                    if (e < n) caxpy((e & 1) ? ac2 : acc, Jreg[e], z[zi]);
+                    caxpy((e & 1) ? ac2 : acc, Jreg[e], z[e < n ? zi : 0]);
                     zi += step; step -= 4;
                 }
             } else {
@@ -190,19 +203,15 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
                 }
             }
             acc.x += ac2.x; acc.y += ac2.y;
-            V d, am = a[m], x = acc;
-            if (fk) { d.x = P.nk.x - P.ak.x; d.y = P.nk.y - P.ak.y; }
-            else {
-                d.x = P.nj.x - P.aj.x; d.y = P.nj.y - P.aj.y;
-                if (y >= 0) {  // the pair {k, y} with k replaced
-                    V dk;
-                    dk.x = P.nk.x - P.ak.x; dk.y = P.nk.y - P.ak.y;
-                    caxpy(x, Jb, cmul(dk, a[y]));
-                }
-                if (m == k) am = P.nk;
-            }
-            const V w = cmulc(am, x);
-            share = d.x * w.x + d.y * w.y;
+            // share = Re[conj(d) conj(a_m) x] = Re[conj(d a_m) x], x = acc, for field j with a_k replaced: the pair {k, y}
+            // changes by dk a_y, and partner k is nk.  d a_m and J a_y wait for no sum
+            const V d = fk ? P.dk : P.dj, am = (!fk && m == k) ? P.nk : a[m], dm = cmul(d, am);
+            V x = acc;
+            const V ay = a[y >= 0 ? y : 0], dk = P.dk;
+            const real tx = Jb * ay.x, ty = Jb * ay.y;  // zero coupling where there is no such pair
+            x.x = fma(dk.x, tx, fma(-dk.y, ty, x.x));
+            x.y = fma(dk.x, ty, fma(dk.y, tx, x.y));
+            share = fma(dm.x, x.x, dm.y * x.y);
         }
         if (!helper) {
 #pragma unroll
@@ -218,7 +227,7 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
                     if (j2 == j) aj = P.nj; else if (j2 == k) aj = P.nk;
                     if (k2 == j) ak = P.nj; else if (k2 == k) ak = P.nk;
                 }
-                prop[((i + 1) & 1) * 2 + lane] = finish_proposal<real>(draws[at], aj, ak);
+                propose(prop[((i + 1) & 1) * 2 + lane], draws[at], aj, ak);
             }
         }
         if (traced) {  // the record of this update (h_j, h_k, B_jk, A_jk) and the state before it
@@ -255,7 +264,7 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
         share = part[(i & 1) * 32];
         for (int w = 1; w < RW; ++w) share += part[(i & 1) * 32 + w];
         const real dH = -cc * share;
-        const bool take = row_accept<real>(dH, beta, P.U);
+        const bool take = row_accept<real>(share, dH, beta, P.test);
         if (traced && tid == 0) {
             const ProposalDraw<real> &D = draws[i & (2 * kRowDraws - 1)];
             double *rec = p.trace + (int64_t)cid * kTraceRec;
@@ -328,6 +337,10 @@ cudaError_t launch_row_pack(bool dbl, const SampleDev *samples, int S, const int
 
 size_t row_smem_bytes(bool dbl, int maxN) { return dbl ? RowSmem<double>(maxN).total : RowSmem<float>(maxN).total; }
 
+// GB300, us per sweep: N = 16, 64 chains FP64 16.7 (268 on J-sharing blocks of 16 chains, 4 SMs busy); N = 64, 1024 chains
+// FP64 856 (2230 on blocks of 8, 4187 of 16), 4096 chains 3460 (6110); N = 128, 512 chains FP64 2990 (10270); N = 18, 168
+// chains FP32 8.0 (17.1); N = 32, 168 chains FP32 14.3 (32).  What is left of an update of few rows is a chain of FP64
+// latencies (about 70 clocks each); a third warp for the random numbers alone gained 5% there and cost as much at FP32.
 // Variants by the largest N: rows of at most 8 or 16 pairs keep their couplings in registers; longer rows load them in
 // eights.  The register budget follows the blocks an SM holds at that N (pair products of 227 KB).
 #define PT_ROW_DISPATCH(T, CALL)                                                                      \
