@@ -93,7 +93,7 @@ def profiled_traffic():
     since the counters were taken."""
     try:
         txt = open(os.path.join(ROOT, "profiles", "sweep_kernel_n256.md")).read()
-        sha = kernel_code_sha(os.path.join(ROOT, "paper_2511_13508_gb300", "csrc", "pt_sweep.cu"))
+        sha = kernel_code_sha(os.path.join(ROOT, "paper_2511_13508_gb300", "csrc", "pt_comb.cu"))
     except OSError:
         return None
     if ("code sha1 prefix `%s`" % sha) not in txt:
@@ -872,7 +872,7 @@ def main(argv=None):
                 "vs_baseline": None, "dtype": "f32", "data": "synthetic", "config": cfg,
                 "roofline": {"bound": "alu", "achieved": r["achieved"], "peak": r["peak"], "unit": "TFLOP/s",
                              "frac": r["achieved"] / r["peak"], "traffic": profiled_traffic(),
-                             "kernel": "sweep_kernel<float,8,11> (8 chains x 11 field warps + 1 copy warp per block)",
+                             "kernel": "comb_sweep_kernel<8,11,1> (8 chains x 11 field warps + 1 copy warp per block)",
                              "kernel_ms_per_launch": r["kms"],
                              "flop_count": "algorithmic: 16 FP32 flops x 4|Q| coupling terms per chain-sweep "
                                            "(87.9 MFLOP at N=256)",

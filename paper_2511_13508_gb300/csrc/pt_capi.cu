@@ -1351,12 +1351,12 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
                 c->max_chunks = std::max(c->max_chunks, lists[s].max_chunks);
                 c->max_cross = std::max(c->max_cross, lists[s].max_cross);
             }
-            RC(dalloc(c, &c->d_chunks, nch));
-            RC(dalloc(c, &c->d_cross, ncr));
-            RC(dalloc(c, &c->d_choff, nco));
-            RC(dalloc(c, &c->d_xoff, nxo));
+            // without room for them the sweep takes the incidence records
+            const bool room = dalloc(c, &c->d_chunks, nch) == PT_OK && dalloc(c, &c->d_cross, ncr) == PT_OK &&
+                              dalloc(c, &c->d_choff, nco) == PT_OK && dalloc(c, &c->d_xoff, nxo) == PT_OK;
+            if (!room) c->d_chunks = nullptr;
             nco = 0;
-            for (int s = 0; s < S; ++s) {
+            for (int s = 0; room && s < S; ++s) {
                 const SampleDev &sd = c->samples[s];
                 const GraphLists &g = lists[s];
                 CK(cudaMemcpy(c->d_chunks + 2 * sd.chunk_off, g.chunks.data(), g.chunks.size() * sizeof(int4), cudaMemcpyHostToDevice));
@@ -1409,7 +1409,9 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     if (c->gfp32) CK(graph_prepare(graph_params(c)));
     if (c->row) {
         c->d_Jrow = dev_alloc(c, (size_t)row_total * c->esize);
-        if (!c->d_Jrow) return bail(fail(c, PT_ENOMEM, "device allocation failed (couplings)"));
+        if (!c->d_Jrow) c->row = false;  // no room for the second store: the J-sharing blocks sweep
+    }
+    if (c->row) {
         CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
         CK(launch_row_pack(c->dbl, c->d_samples, S, c->d_quads, c->d_Jq, c->d_Jrow, c->stream));
         std::vector<int> order(c->n_chains);

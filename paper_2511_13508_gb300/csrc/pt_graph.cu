@@ -775,6 +775,13 @@ __global__ void __launch_bounds__(NT, 1) graph_table_kernel(GraphParams p) {
             }
         }
     }
+    // never leave bulk copies in flight behind an exiting block (only possible after a wait gave up)
+    if (helper && lane == 0 && *abort_flag)
+        for (int n = max(0, total - nbuf); n < total; ++n) {
+            const unsigned long long t0 = global_ns();
+            while (!mbar_try_wait(&lbar[nbuf == 2 ? n & 1 : 0], (uint32_t)(nbuf == 2 ? (n >> 1) & 1 : n & 1)) && global_ns() - t0 < kWaitNs) {
+            }
+        }
     for (int i = tid; i < N * gr.count; i += NT) {
         const int ch = i / N, x = i - ch * N;
         A[i] = amp[x * GC + ch];
@@ -859,10 +866,12 @@ namespace {
 constexpr int kWarpMaxRec = 256;
 constexpr size_t kGraphSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part (the static reduction table aside)
 
-// Whether the pair-table kernel's chunk lists are worth building (their sizes then decide): the products of 4 chains fit.
+// Whether the pair-table kernel's lists are worth building (their sizes then decide): the products of 4 chains and the two
+// lists of an update (32 bytes per four records) fit.
 }  // namespace
 bool graph_table_candidate(int maxN, int max_deg) {
-    return 2 * max_deg > kWarpMaxRec && (size_t)maxN * (maxN - 1) / 2 * 4 * sizeof(float2) < kGraphSmemMax;
+    return 2 * max_deg > kWarpMaxRec &&
+           (size_t)maxN * (maxN - 1) / 2 * 4 * sizeof(float2) + (size_t)2 * max_deg * 8 < kGraphSmemMax;
 }
 namespace {
 // Shape of the pair-table kernel: chains per block, list buffers (two when they fit, so that an update's lists arrive
