@@ -1468,7 +1468,8 @@ int pt_sweep(pt_ctx *c, int64_t n) {
         const int ge = c->learn ? c->learn->global_every : 0;
         for (int e : {cf.swap_every, cf.resync_every, ge})
             if (e > 0) nb = std::min(nb, (d / e + 1) * e);
-        const int seg = (int)std::min<int64_t>(n, nb - d);
+        const int64_t most = std::max(1, (1 << 30) / std::max(1, c->maxN / 2));  // updates of a launch are counted in an int
+        const int seg = (int)std::min<int64_t>({n, nb - d, most});
         const int64_t end = d + seg;
         SegKey k{};
         k.seg = seg;
