@@ -558,7 +558,6 @@ int learn_backward(pt_ctx *c, int rows, const int *cond) {
     w3.M = sh.Dout; w3.N = sh.H; w3.K = rows; w3.mode = kEpiF32;
     w3.D = L.Gr + sh.oW3; w3.strideD = ps; w3.ldd = sh.H;
     w3.err = &c->d_ctl->error;
-    CK(launch_gemm_bf16(w3, c->S, c->stream));
     GemmParams g1 = g;  // dZ1 = (dZ2 W2) * [Z1 > 0]
     g1.A = L.dZ2b; g1.strideA = rc * sh.H; g1.lda = sh.H;
     g1.B = L.W2T; g1.strideB = (int64_t)sh.H * sh.H; g1.ldb = sh.H; g1.K = sh.H;
@@ -567,14 +566,14 @@ int learn_backward(pt_ctx *c, int rows, const int *cond) {
     GemmParams w2 = w3;  // dW2 = dZ2^T H1
     w2.A = L.dZ2T; w2.strideA = rc * sh.H; w2.B = L.H1T; w2.strideB = rc * sh.H;
     w2.M = sh.H; w2.N = sh.H; w2.D = L.Gr + sh.oW2; w2.ldd = sh.H;
-    CK(launch_gemm_bf16(w2, c->S, c->stream));
     GemmParams w1 = w3;  // dW1 = dZ1^T X
     w1.A = L.dZ1T; w1.strideA = rc * sh.H; w1.B = L.XT; w1.strideB = rc * sh.Din;
     w1.M = sh.H; w1.N = sh.Din; w1.D = L.Gr + sh.oW1; w1.ldd = sh.Din;
-    CK(launch_gemm_bf16(w1, c->S, c->stream));
-    CK(launch_colsum(L.dO, rows, sh.Dout, L.Gr + sh.ob3, nullptr, nullptr, 0, c->S, rc * sh.Dout, ps, c->stream));
-    CK(launch_colsum(L.dZ2, rows, sh.H, L.Gr + sh.ob2, nullptr, nullptr, 0, c->S, rc * sh.H, ps, c->stream));
-    CK(launch_colsum(L.dZ1, rows, sh.H, L.Gr + sh.ob1, L.Gr + sh.oC1, cond, sh.ncold, c->S, rc * sh.H, ps, c->stream));
+    const GemmParams ws[3] = {w3, w2, w1};
+    CK(launch_gemm_group(ws, 3, c->S, c->stream));
+    const ColSum cs[3] = {{L.dO, sh.Dout, L.Gr + sh.ob3, nullptr, rc * sh.Dout}, {L.dZ2, sh.H, L.Gr + sh.ob2, nullptr, rc * sh.H},
+                          {L.dZ1, sh.H, L.Gr + sh.ob1, L.Gr + sh.oC1, rc * sh.H}};
+    CK(launch_colsums(cs, 3, rows, cond, sh.ncold, c->S, ps, c->stream));
     return PT_OK;
 }
 

@@ -95,12 +95,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 
 }  // namespace
 
+// (One launch for the three weight gradients, which are independent: 42 us against 56, K = 512, cold caches on GB300.)
+// Products of one launch: block x works on problem i, first[i] <= x < first[i + 1], whose tiles run over M first.
+struct GemmGroup {
+    GemmParams p[kGemmGroup];
+    int first[kGemmGroup];  // of the problems past the last: beyond the grid
+};
+
 // Two-stage pipeline: the copies of chunk c+1 are in flight while the tensor cores work on chunk c.
-__global__ void __launch_bounds__(128, 2) gemm_bf16_tc_kernel(GemmParams p) {
+__global__ void __launch_bounds__(128, 2) gemm_bf16_tc_kernel(const __grid_constant__ GemmGroup grp) {
+    int which = 0;
+    while (which + 1 < kGemmGroup && (int)blockIdx.x >= grp.first[which + 1]) ++which;
+    const GemmParams &p = grp.p[which];
+    const int tile_id = (int)blockIdx.x - grp.first[which], mtiles = (p.M + kGemmM - 1) / kGemmM;
     extern __shared__ __align__(1024) unsigned char gsm[];
     __shared__ uint64_t mbar[2];
     __shared__ uint32_t tmem_base_slot;
-    const int b = blockIdx.z, m0 = blockIdx.x * kGemmM, n0 = blockIdx.y * kGemmNT;
+    const int b = blockIdx.y, m0 = tile_id % mtiles * kGemmM, n0 = tile_id / mtiles * kGemmNT;
     const int N = p.N, K = p.K, NT = min(kGemmNT, N - n0);
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     constexpr uint32_t kStageA = kGemmM * kGemmKC * 2, kStage = kStageA + kGemmNT * kGemmKC * 2;
@@ -177,9 +188,11 @@ __global__ void __launch_bounds__(128, 2) gemm_bf16_tc_kernel(GemmParams p) {
     if (!ok) {
         if (threadIdx.x == 0 && p.err) atomicCAS(p.err, 0, kErrTimeout);
     } else {
-        // epilogue.  Phase 1 (lane = row): warp w reads TMEM lanes 32w..32w+31, 32 columns at a time, applies
-        // bias / conditional bias / gate, writes the transposed BF16 copy (coalesced along rows) and parks the
-        // values in a 32 x 33 shared tile.  Phase 2 (lane = column): row-major FP32 and BF16 stores, coalesced.
+        // Epilogue, 32 columns at a time.  Warp w reads TMEM lanes 32w..32w+31 (lane = row) and parks the values in a
+        // 32 x 33 shared tile; then lane = column: bias, conditional bias or gate, row-major FP32 and BF16 stores; then
+        // lane = row again for the transposed BF16 copy.  Global accesses are coalesced and a tile's gate values (or conditional
+        // biases) are in flight together.  Latency bounds the kernel at these sizes: 16 samples, 512 x 256 outputs, K = 256,
+        // cold caches on GB300: gated 27.8 -> 19.3 us, forward 21.4 -> 17.8, against gate and conditional bias read lane = row.
         float *tile = reinterpret_cast<float *>(gsm) + warp * (32 * 33);
         const int row = m0 + warp * 32 + lane;
         const bool relu = p.mode == kEpiRelu;
@@ -196,34 +209,56 @@ __global__ void __launch_bounds__(128, 2) gemm_bf16_tc_kernel(GemmParams p) {
                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            const bool live = row < p.M;
-            const float *cb = (p.cbias && live)
-                                  ? p.cbias + (int64_t)b * p.strideCbias + (int64_t)p.cond[(int64_t)b * p.strideCond + row] * N
-                                  : nullptr;
-            const float *gt = (p.mode == kEpiGate && live)
-                                  ? p.gate + (int64_t)b * p.strideGate + (int64_t)row * p.ldgate : nullptr;
 #pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                const int col = n0 + c0 + q;
-                float v = __uint_as_float(r[q]);
-                if (p.mode == kEpiGate) {
-                    v = (gt && col < N && gt[col] > 0.f) ? v : 0.f;
-                } else {
-                    if (p.bias && col < N) v += p.bias[(int64_t)b * p.strideBias + col];
-                    if (cb && col < N) v += cb[col];
-                }
-                tile[lane * 33 + q] = v;
-                if (p.HT && live && col < N)
-                    p.HT[(int64_t)b * p.strideHT + (int64_t)col * p.ldht + row] = __float2bfloat16_rn(relu ? fmaxf(v, 0.f) : v);
-            }
+            for (int q = 0; q < 32; ++q) tile[lane * 33 + q] = __uint_as_float(r[q]);
             __syncwarp();
-            const int col = n0 + c0 + lane;
+            const int col = n0 + c0 + lane, colc = min(col, N - 1), row0 = m0 + warp * 32, rows = min(32, p.M - row0);
+            const bool keep = p.HT != nullptr, gated = p.mode == kEpiGate;
+            float ex[32];  // gate or conditional bias of the lane's column, all rows' loads in flight together
+#pragma unroll
+            for (int rr = 0; rr < 32; ++rr) ex[rr] = 0.f;
+            if (gated && p.gate) {
+                const float *gt = p.gate + (int64_t)b * p.strideGate + (int64_t)row0 * p.ldgate + colc;
+#pragma unroll
+                for (int rr = 0; rr < 32; ++rr)
+                    if (rr < rows) ex[rr] = __ldg(gt + (int64_t)rr * p.ldgate);
+            } else if (!gated && p.cbias) {
+                const float *cb = p.cbias + (int64_t)b * p.strideCbias + colc;
+                const int cd = lane < rows ? __ldg(p.cond + (int64_t)b * p.strideCond + row0 + lane) : 0;
+#pragma unroll
+                for (int rr = 0; rr < 32; ++rr) {
+                    const int cr = __shfl_sync(0xffffffffu, cd, rr);
+                    if (rr < rows) ex[rr] = __ldg(cb + (int64_t)cr * N);
+                }
+            }
+            const float bias = p.bias && !gated ? __ldg(p.bias + (int64_t)b * p.strideBias + colc) : 0.f;
+            float *D = p.D && col < N ? p.D + (int64_t)b * p.strideD + (int64_t)row0 * p.ldd + col : nullptr;
+            __nv_bfloat16 *H = p.H && col < N ? p.H + (int64_t)b * p.strideH + (int64_t)row0 * p.ldh + col : nullptr;
+            float val[32];
+#pragma unroll
+            for (int rr = 0; rr < 32; ++rr) val[rr] = tile[rr * 33 + lane];
+#pragma unroll
             for (int rr = 0; rr < 32; ++rr) {
-                const int row2 = m0 + warp * 32 + rr;
-                if (row2 >= p.M || col >= N) continue;
-                const float v = tile[rr * 33 + lane];
-                if (p.D) p.D[(int64_t)b * p.strideD + (int64_t)row2 * p.ldd + col] = v;
-                if (p.H) p.H[(int64_t)b * p.strideH + (int64_t)row2 * p.ldh + col] = __float2bfloat16_rn(relu ? fmaxf(v, 0.f) : v);
+                if (rr >= rows) break;
+                float v = val[rr];
+                if (gated) {
+                    v = ex[rr] > 0.f ? v : 0.f;
+                } else {
+                    if (p.bias) v += bias;
+                    if (p.cbias) v += ex[rr];
+                }
+                if (D) D[(int64_t)rr * p.ldd] = v;
+                if (relu) v = fmaxf(v, 0.f);
+                if (H) H[(int64_t)rr * p.ldh] = __float2bfloat16_rn(v);
+                if (keep) tile[rr * 33 + lane] = v;
+            }
+            if (keep) {
+                __syncwarp();
+                if (row < p.M) {
+                    __nv_bfloat16 *HT = p.HT + (int64_t)b * p.strideHT + (int64_t)(n0 + c0) * p.ldht + row;
+#pragma unroll 8
+                    for (int q = 0; q < min(32, N - (n0 + c0)); ++q) HT[(int64_t)q * p.ldht] = __float2bfloat16_rn(tile[lane * 33 + q]);
+                }
             }
             __syncwarp();
         }
@@ -627,9 +662,20 @@ cudaError_t launch_fused_sampler(const MlpParams &p, const SamplerExtra &sx, int
     return launch_mlp_cluster<true>(p, sx, batch, s);
 }
 
-cudaError_t launch_gemm_bf16(const GemmParams &p, int batch, cudaStream_t s) {
-    if (p.N < 16 || p.N > 256 || (p.N % 16) || p.K < 16 || (p.K % 8) || p.M < 1 || batch < 1)
-        return cudaErrorInvalidValue;
+cudaError_t launch_gemm_bf16(const GemmParams &p, int batch, cudaStream_t s) { return launch_gemm_group(&p, 1, batch, s); }
+
+cudaError_t launch_gemm_group(const GemmParams *ps, int n, int batch, cudaStream_t s) {
+    if (n < 1 || n > kGemmGroup || batch < 1) return cudaErrorInvalidValue;
+    GemmGroup grp{};
+    int tiles = 0;
+    for (int i = 0; i < kGemmGroup; ++i) {
+        grp.first[i] = i < n ? tiles : 0x7fffffff;
+        if (i >= n) continue;
+        const GemmParams &p = ps[i];
+        if (p.N < 16 || p.N > 256 || (p.N % 16) || p.K < 16 || (p.K % 8) || p.M < 1) return cudaErrorInvalidValue;
+        grp.p[i] = p;
+        tiles += (p.M + kGemmM - 1) / kGemmM * ((p.N + kGemmNT - 1) / kGemmNT);
+    }
     constexpr size_t sm = 2 * ((size_t)kGemmM * kGemmKC * 2 + (size_t)kGemmNT * kGemmKC * 2);
     static bool attr_set = false;  // per process; the attribute is a property of the function
     if (!attr_set) {
@@ -637,8 +683,7 @@ cudaError_t launch_gemm_bf16(const GemmParams &p, int batch, cudaStream_t s) {
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    dim3 grid((p.M + kGemmM - 1) / kGemmM, (p.N + kGemmNT - 1) / kGemmNT, batch);
-    gemm_bf16_tc_kernel<<<grid, 128, sm, s>>>(p);
+    gemm_bf16_tc_kernel<<<dim3(tiles, batch), 128, sm, s>>>(grp);
     return cudaGetLastError();
 }
 

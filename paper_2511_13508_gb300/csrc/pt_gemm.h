@@ -38,6 +38,9 @@ struct GemmParams {
 };
 
 cudaError_t launch_gemm_bf16(const GemmParams &p, int batch, cudaStream_t s);
+// Up to kGemmGroup independent products of the same batch in one launch.
+constexpr int kGemmGroup = 3;
+cudaError_t launch_gemm_group(const GemmParams *p, int n, int batch, cudaStream_t s);
 
 // The proposal network's whole forward pass for up to 128 rows per sample in one launch:
 // O = W3 relu(W2 relu(W1 x + b1 + C1[cond]) + b2) + b3, the hidden activations kept in shared memory (BF16)

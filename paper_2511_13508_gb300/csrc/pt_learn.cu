@@ -234,16 +234,22 @@ cudaError_t launch_density(const DensityParams &p, int S, cudaStream_t s) {
 // waited for the one before: 105 us on GB300 for 512 rows of 256 columns and 16 samples; 9 us now.)
 constexpr int kColBatch = 32, kColThreads = 32, kColCond = 64;
 
+// The layers' sums are independent: one launch, block x on columns [32 x', 32 x' + 32) of its layer.
+struct ColGroup {
+    ColSum p[kColGroup];
+    int first[kColGroup];
+    const int *cond;
+    int rows, ncond;
+    int64_t strideGrad;
+};
+
 template <bool kC>
-__global__ void __launch_bounds__(kColThreads) colsum_kernel(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond,
-                                                             int ncond, int64_t strideZ, int64_t strideGrad, int64_t strideCond) {
-    __shared__ float sC[kC ? kColCond : 1][kColThreads];
-    const int s = blockIdx.y, lane = threadIdx.x, col = blockIdx.x * kColThreads + lane;
+__device__ __forceinline__ void colsum_body(const ColGroup &g, const ColSum &p, int s, int col, float (*sC)[kColThreads]) {
+    const int lane = threadIdx.x, rows = g.rows, cols = p.cols;
     if (kC)
-        for (int i = 0; i < ncond; ++i) sC[i][lane] = 0.f;
-    if (col >= cols) return;
-    const float *z = dZ + s * strideZ + col;
-    const int *cs = kC ? cond + s * strideCond : nullptr;
+        for (int i = 0; i < g.ncond; ++i) sC[i][lane] = 0.f;
+    const float *z = p.dZ + s * p.strideZ + col;
+    const int *cs = kC ? g.cond + (int64_t)s * rows : nullptr;
     float acc = 0.f;
     for (int r0 = 0; r0 < rows; r0 += kColBatch) {
         float v[kColBatch];
@@ -260,32 +266,46 @@ __global__ void __launch_bounds__(kColThreads) colsum_kernel(const float *dZ, in
             if (kC) sC[k[e]][lane] += v[e];
         }
     }
-    db[s * strideGrad + col] = acc;
+    p.db[s * g.strideGrad + col] = acc;
     if (kC)
-        for (int i = 0; i < ncond; ++i) dC[s * strideGrad + (int64_t)i * cols + col] = sC[i][lane];
+        for (int i = 0; i < g.ncond; ++i) p.dC[s * g.strideGrad + (int64_t)i * cols + col] = sC[i][lane];
 }
 
-// More conditions than shared memory holds: dC straight in global memory (zeroed by the caller).
-__global__ void colsum_wide_kernel(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond, int64_t strideZ,
-                                   int64_t strideGrad, int64_t strideCond) {
-    const int s = blockIdx.y, col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= cols) return;
-    const float *z = dZ + s * strideZ;
-    float acc = 0.f;
-    for (int r = 0; r < rows; ++r) {
-        const float v = z[(int64_t)r * cols + col];
-        acc += v;
-        dC[s * strideGrad + (int64_t)cond[s * strideCond + r] * cols + col] += v;
+__global__ void __launch_bounds__(kColThreads) colsum_kernel(const __grid_constant__ ColGroup g) {
+    __shared__ float sC[kColCond][kColThreads];
+    int which = 0;
+    while (which + 1 < kColGroup && (int)blockIdx.x >= g.first[which + 1]) ++which;
+    const ColSum &p = g.p[which];
+    const int s = blockIdx.y, col = ((int)blockIdx.x - g.first[which]) * kColThreads + threadIdx.x;
+    if (col >= p.cols) return;
+    if (!p.dC) {
+        colsum_body<false>(g, p, s, col, sC);
+    } else if (g.ncond <= kColCond) {
+        colsum_body<true>(g, p, s, col, sC);
+    } else {  // more conditions than shared memory holds: dC straight in global memory
+        const float *z = p.dZ + s * p.strideZ;
+        float acc = 0.f;
+        for (int r = 0; r < g.rows; ++r) {
+            const float v = z[(int64_t)r * p.cols + col];
+            acc += v;
+            p.dC[s * g.strideGrad + (int64_t)g.cond[(int64_t)s * g.rows + r] * p.cols + col] += v;
+        }
+        p.db[s * g.strideGrad + col] = acc;
     }
-    db[s * strideGrad + col] = acc;
 }
 
-cudaError_t launch_colsum(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond, int ncond, int S,
-                          int64_t strideZ, int64_t strideGrad, cudaStream_t s) {
-    const dim3 grid((cols + kColThreads - 1) / kColThreads, S);
-    if (!dC) colsum_kernel<false><<<grid, kColThreads, 0, s>>>(dZ, rows, cols, db, dC, cond, 0, strideZ, strideGrad, rows);
-    else if (ncond <= kColCond) colsum_kernel<true><<<grid, kColThreads, 0, s>>>(dZ, rows, cols, db, dC, cond, ncond, strideZ, strideGrad, rows);
-    else colsum_wide_kernel<<<grid, kColThreads, 0, s>>>(dZ, rows, cols, db, dC, cond, strideZ, strideGrad, rows);
+cudaError_t launch_colsums(const ColSum *p, int n, int rows, const int *cond, int ncond, int S, int64_t strideGrad, cudaStream_t s) {
+    if (n < 1 || n > kColGroup) return cudaErrorInvalidValue;
+    ColGroup g{};
+    g.cond = cond; g.rows = rows; g.ncond = ncond; g.strideGrad = strideGrad;
+    int blocks = 0;
+    for (int i = 0; i < kColGroup; ++i) {
+        g.first[i] = i < n ? blocks : 0x7fffffff;
+        if (i >= n) continue;
+        g.p[i] = p[i];
+        blocks += (p[i].cols + kColThreads - 1) / kColThreads;
+    }
+    colsum_kernel<<<dim3(blocks, S), kColThreads, 0, s>>>(g);
     return cudaGetLastError();
 }
 

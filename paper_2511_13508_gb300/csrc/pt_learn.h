@@ -80,9 +80,16 @@ struct DensityParams {
 };
 cudaError_t launch_density(const DensityParams &p, int S, cudaStream_t s);
 
-// Bias gradients: db[col] = sum_rows dZ[row][col]; dC[cond[row]][col] += dZ[row][col] (optional)
-cudaError_t launch_colsum(const float *dZ, int rows, int cols, float *db, float *dC, const int *cond, int ncond, int S,
-                          int64_t strideZ, int64_t strideGrad, cudaStream_t s);
+// Bias gradients of up to three layers in one launch: db[col] = sum_rows dZ[row][col]; dC[cond[row]][col] += dZ[row][col]
+// (optional; zeroed by the caller).
+constexpr int kColGroup = 3;
+struct ColSum {
+    const float *dZ;  // [S][strideZ], rows of `cols`
+    int cols;
+    float *db, *dC;  // [S][strideGrad]
+    int64_t strideZ;
+};
+cudaError_t launch_colsums(const ColSum *p, int n, int rows, const int *cond, int ncond, int S, int64_t strideGrad, cudaStream_t s);
 
 // Adam on [S][psize] parameters (grad G already averaged).
 cudaError_t launch_adam(float *P, const float *G, float *m, float *v, size_t n, float lr, float b1, float b2,
