@@ -1,7 +1,9 @@
 // pt_graph.cu -- FP32 sweep and energy kernels for explicit interaction lists (the random-frequency
 // mode-locked graph of arXiv 2511.13508, Sec. II.C, or any list of quadruplets).
 //
-// One thread block per group of up to 8 chains of one disorder sample.  A lane is (chain c, worker w):
+// Three sweeps, by the number of records of an update and N (graph_variant below): one chain per block of two warps for
+// few records, a table of pair products shared by the records of a dense graph, and, for the rest and for the energies,
+// one thread block per group of up to 8 chains of one disorder sample.  In that last one a lane is (chain c, worker w):
 // the 128 workers of the block split the quadruplets that hold the updated modes j or k, and the 8
 // lanes of a worker read each incidence record once for their 8 chains.  An incidence record of mode l
 // is (the other three modes in position order, (q << 2) | position of l) with its coupling alongside,
@@ -863,15 +865,21 @@ __global__ void __launch_bounds__(kGThreads) graph_energy_kernel(GraphParams p) 
 }
 
 namespace {
-constexpr int kWarpMaxRec = 256;
+// Records of an update (twice the largest degree) up to which a chain gets a block of its own (graph_warp_kernel): against the
+// pair table with 8 chains per block, and against what remains where that table does not fit.  GB300, us per sweep, own
+// block / other kernel.  Table: sparse N = 48, 1024 and 4096 chains, 120 records 27 / 40 and 75 / 143, 186 39 / 42 and
+// 112 / 150, 268 50 / 42 and 144 / 151, 352 67 / 43 and 192 / 157.  Table of 4 chains, N = 96: 190 76 / 129 and 217 / 439,
+// 314 113 / 138 and 331 / 470.  Group kernel, N = 256: 80 91 / 292 and 275 / 1143, 272 241 / 314 and 724 / 1237, 418
+// 380 / 347 and 1145 / 1364.
+constexpr int kWarpMaxRec = 256, kWarpMaxAlone = 352;
 constexpr size_t kGraphSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part (the static reduction table aside)
 
 // Whether the pair-table kernel's lists are worth building (their sizes then decide): the products of 4 chains and the two
 // lists of an update (32 bytes per four records) fit.
 }  // namespace
 bool graph_table_candidate(int maxN, int max_deg) {
-    return 2 * max_deg > kWarpMaxRec &&
-           (size_t)maxN * (maxN - 1) / 2 * 4 * sizeof(float2) + (size_t)2 * max_deg * 8 < kGraphSmemMax;
+    const size_t pairs = (size_t)maxN * (maxN - 1) / 2 * sizeof(float2), lists = (size_t)2 * max_deg * 8;
+    return 2 * max_deg > (8 * pairs + lists < kGraphSmemMax ? kWarpMaxRec : kWarpMaxAlone) && 4 * pairs + lists < kGraphSmemMax;
 }
 namespace {
 // Shape of the pair-table kernel: chains per block, list buffers (two when they fit, so that an update's lists arrive
@@ -896,8 +904,9 @@ bool table_shape(const GraphParams &p, TabShape *out) {
 }
 int graph_variant(const GraphParams &p) {
     TabShape t;
-    if (2 * p.max_deg <= kWarpMaxRec) return kWarp;
-    if (p.chunks && table_shape(p, &t)) return kTable;
+    const bool table = p.chunks && table_shape(p, &t);
+    if (2 * p.max_deg <= (table && t.GC == 8 ? kWarpMaxRec : kWarpMaxAlone)) return kWarp;
+    if (table) return kTable;
     if (graph_smem(p.maxN, 2 * p.max_deg).total <= kGraphSmemMax) return kStage;
     return kPlain;
 }

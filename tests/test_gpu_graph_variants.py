@@ -26,6 +26,7 @@ CASES = [
     ("random", [4, 6], 0, 1, 3), ("random", [12, 16], 0, 2, 5), ("random", [18], 0, 2, 4), ("random", [32, 20, 26], 0, 2, 3),
     ("random", [64, 34], 0, 1, 9), ("random", [72], 0, 1, 4), ("random", [80], 0, 1, 7), ("random", [96, 64], 0, 1, 5),
     ("sparse", [64, 40], 4, 2, 5), ("sparse", [256], 16, 1, 3), ("sparse", [128], 40, 2, 2), ("sparse", [128], 70, 1, 3),
+    ("sparse", [256], 100, 1, 3), ("sparse", [96], 110, 1, 3), ("sparse", [256], 160, 1, 3), ("random", [128], 0, 1, 2),
 ]
 
 
