@@ -136,44 +136,81 @@ __device__ __forceinline__ size_t sliced_canonical(size_t n, size_t k, size_t N,
     return ((n / NS) * (K / 8) + k / 8) * NS * 8 + (n % NS) * 8 + k % 8;
 }
 
-__global__ void cast_kernel(CastParams p) {
+// A block converts a 32 x 32 tile of a weight matrix: read and written along k, then from shared memory along n for the
+// transposed copy and in 16-byte groups for the canonical one.  (An element per thread, each copy written where it fell, spread
+// a warp's stores over 32 lines.  N = 64, 16 samples, cold caches on GB300: 24.9 -> 12.4 us.)
+constexpr int kCastT = 32;
+__global__ void __launch_bounds__(256) cast_kernel(CastParams p) {
+    __shared__ __nv_bfloat16 tile[kCastT][kCastT + 2];
     const LearnShape &sh = p.sh;
     const int s = blockIdx.y;
-    const float *P = p.P + (size_t)s * sh.psize;
-    const size_t n1 = (size_t)sh.H * sh.Din, n2 = (size_t)sh.H * sh.H, n3 = (size_t)sh.Dout * sh.H;
-    for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n1 + n2 + n3; i += gridDim.x * blockDim.x) {
-        if (i < n1) {
-            const __nv_bfloat16 w = __float2bfloat16_rn(P[sh.oW1 + i] * p.M1[i]);
-            p.W1[s * n1 + i] = w;
-            p.W1c[s * n1 + sliced_canonical(i / sh.Din, i % sh.Din, sh.H, sh.Din)] = w;
-        } else if (i < n1 + n2) {
-            const size_t j = i - n1;
-            const __nv_bfloat16 w = __float2bfloat16_rn(P[sh.oW2 + j] * p.M2[j]);
-            p.W2[s * n2 + j] = w;
-            const size_t h2 = j / sh.H, h1 = j % sh.H;
-            p.W2T[s * n2 + h1 * sh.H + h2] = w;
-            p.W2c[s * n2 + sliced_canonical(h2, h1, sh.H, sh.H)] = w;
-        } else {
-            const size_t j = i - n1 - n2;
-            const __nv_bfloat16 w = __float2bfloat16_rn(P[sh.oW3 + j] * p.M3[j]);
-            p.W3[s * n3 + j] = w;
-            const size_t o = j / sh.H, h = j % sh.H;
-            p.W3T[s * n3 + h * sh.Dout + o] = w;
-            p.W3c[s * n3 + sliced_canonical(o, h, sh.Dout, sh.H)] = w;
+    auto tiles = [](int n, int k) { return (n + kCastT - 1) / kCastT * ((k + kCastT - 1) / kCastT); };
+    const int t1 = tiles(sh.H, sh.Din), t2 = tiles(sh.H, sh.H);
+    int t = blockIdx.x, N = sh.H, K = sh.Din;
+    const float *P = p.P + (size_t)s * sh.psize + sh.oW1, *M = p.M1;
+    __nv_bfloat16 *W = p.W1, *WT = nullptr, *Wc = p.W1c;
+    if (t >= t1 + t2) {
+        t -= t1 + t2;
+        N = sh.Dout; K = sh.H; P = p.P + (size_t)s * sh.psize + sh.oW3; M = p.M3; W = p.W3; WT = p.W3T; Wc = p.W3c;
+    } else if (t >= t1) {
+        t -= t1;
+        K = sh.H; P = p.P + (size_t)s * sh.psize + sh.oW2; M = p.M2; W = p.W2; WT = p.W2T; Wc = p.W2c;
+    }
+    const int ktiles = (K + kCastT - 1) / kCastT, n0 = t / ktiles * kCastT, k0 = t % ktiles * kCastT;
+    const size_t at = (size_t)s * N * K;
+    const int x = threadIdx.x % kCastT, y = threadIdx.x / kCastT;
+    for (int r = y; r < kCastT; r += 256 / kCastT) {
+        const int n = n0 + r, k = k0 + x;
+        if (n >= N || k >= K) continue;
+        const size_t i = (size_t)n * K + k;
+        const __nv_bfloat16 w = __float2bfloat16_rn(P[i] * M[i]);
+        W[at + i] = w;
+        tile[r][x] = w;
+    }
+    __syncthreads();
+    if (WT)
+        for (int r = y; r < kCastT; r += 256 / kCastT)
+            if (n0 + x < N && k0 + r < K) WT[at + (size_t)(k0 + r) * N + n0 + x] = tile[x][r];
+    if (y < kCastT / 8) {  // K % 8 == 0
+        const int n = n0 + x, k = k0 + 8 * y;
+        if (n < N && k < K) {
+            __align__(16) __nv_bfloat16 g[8];
+            for (int e = 0; e < 8; ++e) g[e] = tile[x][8 * y + e];
+            *reinterpret_cast<uint4 *>(Wc + at + sliced_canonical(n, k, N, K)) = *reinterpret_cast<const uint4 *>(g);
         }
     }
 }
 
 cudaError_t launch_cast(const CastParams &p, cudaStream_t s) {
-    dim3 grid(128, p.sh.S);
+    auto tiles = [](int n, int k) { return (n + kCastT - 1) / kCastT * ((k + kCastT - 1) / kCastT); };
+    const dim3 grid(tiles(p.sh.H, p.sh.Din) + tiles(p.sh.H, p.sh.H) + tiles(p.sh.Dout, p.sh.H), p.sh.S);
     cast_kernel<<<grid, 256, 0, s>>>(p);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------------
-// log q per row and the gradient of mean(-log q) with respect to the outputs (mu, log sigma, m, rho_raw)
-__global__ void density_kernel(DensityParams p) {
-    const int s = blockIdx.y, row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
+// Transposed BF16 copies of R rows (a warp each): collected as t[column][row] in shared memory and written R / 8 pieces of 16
+// bytes a column, where two bytes per row and column would each open a sector of their own.
+constexpr int kTrRows = 16, kTrCols = 4 * 64;
+template <int R>
+__device__ __forceinline__ void write_transposed(__nv_bfloat16 (*t)[R + 2], __nv_bfloat16 *out, int cols, int64_t ld) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < cols * (R / 8); i += blockDim.x) {
+        const int col = i / (R / 8), h = i % (R / 8);
+        __align__(16) __nv_bfloat16 g[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) g[e] = t[col][8 * h + e];
+        *reinterpret_cast<uint4 *>(out + (int64_t)col * ld + 8 * h) = *reinterpret_cast<const uint4 *>(g);
+    }
+}
+
+// log q per row and the gradient of mean(-log q) with respect to the outputs (mu, log sigma, m, rho_raw).  A warp per row: R = 1
+// row per block spreads the few rows of a round of moves over the SMs; R = 16 in training, whose transposed gradient then
+// leaves in pieces of 16 bytes (8192 rows of 64 modes, cold caches on GB300: 29.5 -> 15.9 us).
+template <int R>
+__global__ void __launch_bounds__(32 * R) density_kernel(DensityParams p) {
+    __shared__ __nv_bfloat16 tr[R > 1 ? kTrCols : 1][R + 2];
+    const int s = blockIdx.y, row = blockIdx.x * R + threadIdx.x / 32, lane = threadIdx.x % 32;
     if (row >= p.rows_per_sample) return;
     const int N = p.N;
     const int64_t grow = (int64_t)s * p.rows_per_sample + row;
@@ -212,18 +249,22 @@ __global__ void density_kernel(DensityParams p) {
                 if (p.dO) p.dO[orow * p.Dout + col] = d;
                 const __nv_bfloat16 b = __float2bfloat16_rn(d);
                 if (p.dOb) p.dOb[orow * p.Dout + col] = b;
-                if (p.dOT) p.dOT[((int64_t)s * p.Dout + col) * p.lddt + row] = b;
+                if (R > 1) tr[col][threadIdx.x / 32] = b;
+                else if (p.dOT) p.dOT[((int64_t)s * p.Dout + col) * p.lddt + row] = b;
             }
         }
     }
     lq = warp_sumd(lq);
     if (lane == 0) p.logq[grow] = lq;
+    if constexpr (R > 1) write_transposed<R>(tr, p.dOT + (int64_t)s * p.Dout * p.lddt + blockIdx.x * R, p.Dout, p.lddt);
 }
 
 cudaError_t launch_density(const DensityParams &p, int S, cudaStream_t s) {
     if (p.rows_per_sample <= 0) return cudaSuccess;
-    dim3 grid(p.rows_per_sample, S);  // one row (warp) per block
-    density_kernel<<<grid, 32, 0, s>>>(p);
+    if (p.dOT && p.rows_per_sample % kTrRows == 0 && p.lddt % 8 == 0 && p.Dout <= kTrCols)
+        density_kernel<kTrRows><<<dim3(p.rows_per_sample / kTrRows, S), 32 * kTrRows, 0, s>>>(p);
+    else
+        density_kernel<1><<<dim3(p.rows_per_sample, S), 32, 0, s>>>(p);
     return cudaGetLastError();
 }
 
@@ -338,9 +379,11 @@ cudaError_t launch_adam(float *P, const float *G, float *m, float *v, size_t n, 
 }
 
 // ------------------------------------------------------------------------------------------------
-__global__ void gather_kernel(GatherParams p) {
-    const int s = blockIdx.y, row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
-    if (row >= p.rows) return;
+// A batch of training rows, a warp each, the transposed copy as in density_kernel (8192 rows of 192 features, cold caches on GB300: 19.2 ->
+// 7.4 us).
+__global__ void __launch_bounds__(32 * kTrRows) gather_kernel(GatherParams p) {
+    __shared__ __nv_bfloat16 tr[kTrCols][kTrRows + 2];
+    const int s = blockIdx.y, row = blockIdx.x * kTrRows + threadIdx.x / 32, lane = threadIdx.x % 32;
     const int N = p.N;
     const u32x4 w = draw(p.seed, (uint32_t)s, p.step, (uint32_t)row, kTagBatch);
     const int idx = (int)(((uint64_t)w.x * (uint64_t)p.ndata) >> 32);
@@ -356,18 +399,19 @@ __global__ void gather_kernel(GatherParams p) {
             const int fi = 3 * k + c;
             const __nv_bfloat16 b = __float2bfloat16_rn(f[c]);
             p.X[xrow * p.Din + fi] = b;
-            p.XT[((int64_t)s * p.Din + fi) * p.ldxt + row] = b;
+            tr[fi][threadIdx.x / 32] = b;
         }
     }
     if (lane == 0) {
         p.raw.extra[dst] = p.dextra[src];
         p.raw.cond[dst] = p.dcond[src];
     }
+    write_transposed<kTrRows>(tr, p.XT + (int64_t)s * p.Din * p.ldxt + blockIdx.x * kTrRows, p.Din, p.ldxt);
 }
 
 cudaError_t launch_gather(const GatherParams &p, int S, cudaStream_t s) {
-    dim3 grid((p.rows + 3) / 4, S);
-    gather_kernel<<<grid, 128, 0, s>>>(p);
+    if (p.rows % kTrRows || p.ldxt % 8 || p.Din > kTrCols) return cudaErrorInvalidValue;  // batches are multiples of 128
+    gather_kernel<<<dim3(p.rows / kTrRows, S), 32 * kTrRows, 0, s>>>(p);
     return cudaGetLastError();
 }
 
