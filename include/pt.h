@@ -137,8 +137,8 @@ int pt_fmc_graph(int N, const double *omega, double gamma, int32_t *quads, int64
  * the four modes distinct and < N[s]) and the couplings J[q_offsets[s] .. q_offsets[s+1]) (q_offsets[0] = 0);
  * every N[s] even, 4..2048.
  * Runs on the quadruplet-list paths: PT_PREC_FP64_PLAIN (one thread block per chain, FP64) or PT_PREC_FP32
- * (one thread block per 8 chains of a sample, which read each quadruplet once for all 8; FP32 products,
- * FP64 energies); PT_EUNSUPPORTED for PT_PREC_FP64.  pt_fields and pt_autotune are unsupported on these
+ * (FP32 products, FP64 energies; a block per chain where an update touches few quadruplets, else per 8 chains of a
+ * sample, which read each quadruplet once for all 8); PT_EUNSUPPORTED for PT_PREC_FP64.  pt_fields and pt_autotune are unsupported on these
  * paths.  PT_EINVAL for a bad index or offsets.  The caller keeps ownership of the arrays. */
 int pt_create_graph(pt_ctx **out, const pt_config *cfg, int S, const int32_t *N, const int32_t *quads,
                     const double *J, const int64_t *q_offsets, int n_T, const double *temps, int replicas,
