@@ -6,7 +6,7 @@
 //
 // One thread block computes a 128 x 64 tile with the accumulator in tensor memory: the
 // operands are staged by asynchronous copies (cp.async, zero-filled outside the matrix) in shared memory
-// in the canonical K-major no-swizzle layout (8 x 16-byte core matrices), two stages of K = 128 so that the
+// in the canonical K-major no-swizzle layout (8 x 16-byte core matrices), two stages of K = 96 so that the
 // copies of the next chunk overlap the MMAs of this one; one elected thread issues tcgen05.mma (M = 128,
 // N = 64, K = 16 per instruction) and commits to the stage's mbarrier; four warps read the accumulator back
 // with tcgen05.ld (warp w owns lanes 32w..32w+31) and transpose it through shared memory so that every
@@ -24,8 +24,10 @@ namespace ptgb {
 namespace {
 
 constexpr int kGemmM = 128;   // rows per thread block (= TMEM lanes)
-constexpr int kGemmKC = 128;  // K per pipeline stage (8 MMAs of K = 16)
-constexpr int kGemmNT = 64;   // output columns per thread block (the MMA's N); two stages of 48 KB
+// K per pipeline stage (6 MMAs of K = 16).  Two stages take 72 KB, so that three blocks share an SM and the weight gradients'
+// 352 blocks run at once: four training steps 927 us with 128 (two blocks), 897 with 96, 915 with 64 (four) on GB300.
+constexpr int kGemmKC = 96;
+constexpr int kGemmNT = 64;   // output columns per thread block (the MMA's N); two stages of 36 KB
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -103,7 +105,7 @@ struct GemmGroup {
 };
 
 // Two-stage pipeline: the copies of chunk c+1 are in flight while the tensor cores work on chunk c.
-__global__ void __launch_bounds__(128, 2) gemm_bf16_tc_kernel(const __grid_constant__ GemmGroup grp) {
+__global__ void __launch_bounds__(128, 3) gemm_bf16_tc_kernel(const __grid_constant__ GemmGroup grp) {
     int which = 0;
     while (which + 1 < kGemmGroup && (int)blockIdx.x >= grp.first[which + 1]) ++which;
     const GemmParams &p = grp.p[which];
