@@ -3,6 +3,7 @@
 #include <cstdint>
 #include "pt_common.cuh"
 #include "pt_kernels.h"
+#include "pt_rules.h"
 
 namespace ptgb {
 
@@ -61,8 +62,9 @@ cudaError_t launch_init(const InitParams &p, int n_chains, cudaStream_t s) {
 template <typename V>
 __global__ void canon_kernel(const SampleDev *samples, const int *chain_sample, const int *label, int nT, const V *a, double2 *a_out,
                              int64_t lo, int64_t hi, const double *E, double *E_out, int n_chains) {
-    const int slot = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (slot >= n_chains) return;
+    const int64_t warp = grid_warp(blockIdx.x, blockDim.x, threadIdx.x);
+    if (warp >= n_chains) return;
+    const int slot = (int)warp, lane = threadIdx.x & 31;
     const SampleDev sd = samples[chain_sample[slot]];
     const int at = (slot - sd.chain0) / nT * nT + label[slot];
     if (E && lane == 0) E_out[sd.chain0 + at] = E[slot];
