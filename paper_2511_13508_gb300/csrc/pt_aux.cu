@@ -163,23 +163,26 @@ cudaError_t launch_swap(const SwapParams &p, cudaStream_t s) {
 // 5 measurements of 4 replicas at N = 18 on GB300, latency of the reductions.)
 constexpr int kMeasWarps = 8, kMeasBatch = 32;
 
-template <typename V> __global__ void __launch_bounds__(kMeasWarps * 32) measure_kernel(MeasureParams p) {
+// I counts the tasks: int, or int64_t where all measurements together have more than 2^30.
+template <typename V, typename I> __global__ void __launch_bounds__(kMeasWarps * 32) measure_kernel(MeasureParams p) {
     __shared__ double res[kMeasBatch][6];  // chain: E, Y2, Y4, I; pair: q
     const int s = blockIdx.x / p.nT, t = blockIdx.x % p.nT, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const SampleDev sd = p.samples[s];
-    const int N = sd.N, R = p.R, pairs = R * (R - 1) / 2, per = R + pairs, total = (p.n_snap + (p.live ? 1 : 0)) * per;
+    const int N = sd.N, R = p.R;
+    const I per = (I)measure_tasks(R), total = (p.n_snap + (p.live ? 1 : 0)) * per;
     const int *perm = p.perm + (int64_t)s * R * p.nT;
     double *st = p.stat + ((int64_t)s * p.nT + t) * 7, *qs = p.qstat + ((int64_t)s * p.nT + t) * 5;
     unsigned long long *h = p.qhist + ((int64_t)s * p.nT + t) * 201;
-    for (int b0 = 0; b0 < total; b0 += kMeasBatch) {
-        const int n = min(kMeasBatch, total - b0);
+    for (I b0 = 0; b0 < total; b0 += kMeasBatch) {
+        const int n = (int)min((I)kMeasBatch, total - b0);
         for (int i = warp; i < n; i += kMeasWarps) {
-            const int kk = (b0 + i) / per, task = (b0 + i) - kk * per;
+            const int kk = (int)((b0 + i) / per);
+            const I task = (b0 + i) - kk * per;
             const bool live = kk == p.n_snap;
             const V *a = live ? reinterpret_cast<const V *>(p.a) : reinterpret_cast<const V *>(p.snap_a) + (int64_t)kk * p.a_total;
             const double *E = live ? p.E : p.snap_E + (int64_t)kk * p.n_chains;
             if (task < R) {
-                const int slot = perm[task * p.nT + t];
+                const int slot = perm[(int)task * p.nT + t];
                 const V *x = a + sd.a_off + (int64_t)(slot - sd.chain0) * N;
                 double i2 = 0.0, i4 = 0.0, i8 = 0.0;
                 for (int k = lane; k < N; k += 32) {
@@ -194,9 +197,8 @@ template <typename V> __global__ void __launch_bounds__(kMeasWarps * 32) measure
                 }
                 if (lane == 0) { res[i][0] = E[slot]; res[i][1] = i4 / (i2 * i2); res[i][2] = i8 / (i4 * i4); res[i][3] = i2; }
             } else {
-                int r1 = 0, left = task - R;  // the left-th pair r1 < r2
-                while (left >= R - 1 - r1) { left -= R - 1 - r1; ++r1; }
-                const int r2 = r1 + 1 + left;
+                int r1, r2;
+                replica_pair(task - R, R, &r1, &r2);
                 const V *x = a + sd.a_off + (int64_t)(perm[r1 * p.nT + t] - sd.chain0) * N;
                 const V *y = a + sd.a_off + (int64_t)(perm[r2 * p.nT + t] - sd.chain0) * N;
                 double d = 0.0;
@@ -239,8 +241,12 @@ template <typename V> __global__ void __launch_bounds__(kMeasWarps * 32) measure
 
 cudaError_t launch_measure(const MeasureParams &p, cudaStream_t s) {
     if (p.n_snap <= 0 && !p.live) return cudaSuccess;
-    if (p.dbl) measure_kernel<double2><<<p.S * p.nT, kMeasWarps * 32, 0, s>>>(p);
-    else measure_kernel<float2><<<p.S * p.nT, kMeasWarps * 32, 0, s>>>(p);
+    const int grid = p.S * p.nT;
+    const bool wide = (p.n_snap + (p.live ? 1 : 0)) * measure_tasks(p.R) > (1 << 30);
+    if (wide && p.dbl) measure_kernel<double2, int64_t><<<grid, kMeasWarps * 32, 0, s>>>(p);
+    else if (wide) measure_kernel<float2, int64_t><<<grid, kMeasWarps * 32, 0, s>>>(p);
+    else if (p.dbl) measure_kernel<double2, int><<<grid, kMeasWarps * 32, 0, s>>>(p);
+    else measure_kernel<float2, int><<<grid, kMeasWarps * 32, 0, s>>>(p);
     return cudaGetLastError();
 }
 

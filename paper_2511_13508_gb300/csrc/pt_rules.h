@@ -1,6 +1,7 @@
 // pt_rules.h -- index and scheduling arithmetic of the kernels and their launchers, free of CUDA so that a host compiler
 // takes it too (tests/test_rules_host.py runs it at sizes no GPU test reaches).
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 #ifdef __CUDACC__
@@ -15,6 +16,26 @@ namespace ptgb {
 // a context may hold 2^28 chains.
 PT_HD inline int64_t grid_warp(unsigned block, unsigned block_threads, unsigned thread) {
     return (int64_t)block * (block_threads / 32u) + thread / 32u;
+}
+
+// Tasks of one measurement of a (sample, temperature) with R replicas: the R chains, then the R (R - 1) / 2 replica pairs.
+// From R = 65536 on they pass 2^31; with several measurements at once, earlier.
+PT_HD inline int64_t measure_tasks(int R) { return R + (int64_t)R * (R - 1) / 2; }
+
+// The at-th pair r1 < r2 of R replicas, in the order (0, 1), (0, 2), ..., (1, 2), ...  Row r starts at r (2R - r - 1) / 2; a few
+// replicas are stepped through, for more the quadratic gives the row to within rounding.
+PT_HD inline void replica_pair(int64_t at, int R, int *r1, int *r2) {
+    auto row = [R](int64_t r) { return r * (2 * (int64_t)R - r - 1) / 2; };
+    int64_t r = 0;
+    if (R > 64) {
+        const double b = 2.0 * R - 1.0, d = b * b - 8.0 * (double)at;
+        r = (int64_t)(0.5 * (b - sqrt(d > 0.0 ? d : 0.0)));
+        if (r > R - 2) r = R - 2;
+        while (r > 0 && row(r) > at) --r;
+    }
+    while (row(r + 1) <= at) ++r;
+    *r1 = (int)r;
+    *r2 = (int)(r + 1 + (at - row(r)));
 }
 
 }  // namespace ptgb

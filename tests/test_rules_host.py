@@ -12,6 +12,8 @@ SHIM = r"""
 using namespace ptgb;
 extern "C" {
 int64_t grid_warp_(unsigned b, unsigned n, unsigned t) { return grid_warp(b, n, t); }
+int64_t measure_tasks_(int R) { return measure_tasks(R); }
+void replica_pair_(int64_t at, int R, int *r1, int *r2) { replica_pair(at, R, r1, r2); }
 }
 """
 
@@ -24,7 +26,8 @@ def rules(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2511_13508_gb300", "csrc"),
                     str(d / "shim.cpp"), "-o", so], check=True)
     L = ctypes.CDLL(so)
-    L.grid_warp_.restype = ctypes.c_int64
+    L.grid_warp_.restype = L.measure_tasks_.restype = ctypes.c_int64
+    L.replica_pair_.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
     return L
 
 
@@ -33,3 +36,27 @@ def test_a_warp_per_chain_reaches_every_chain(rules, chain):
     """Blocks of 8 warps: chain c is warp c of the grid, up to the 2^28 chains of a context."""
     for lane in (0, 31):
         assert rules.grid_warp_(chain // 8, 256, chain % 8 * 32 + lane) == chain
+
+
+def _pair(rules, at, R):
+    a, b = ctypes.c_int(), ctypes.c_int()
+    rules.replica_pair_(at, R, ctypes.byref(a), ctypes.byref(b))
+    return a.value, b.value
+
+
+@pytest.mark.parametrize("R", [2, 3, 63, 64, 65, 66, 130])
+def test_replica_pairs_come_in_order(rules, R):
+    pairs = [(i, j) for i in range(R) for j in range(i + 1, R)]
+    assert rules.measure_tasks_(R) == R + len(pairs)
+    assert [_pair(rules, n, R) for n in range(len(pairs))] == pairs
+
+
+@pytest.mark.parametrize("R", [46340, 46341, 65535, 65536, 70000, (1 << 24) + 1, 1 << 28])
+def test_replica_pairs_of_very_many_replicas(rules, R):
+    """Where the count of pairs passes 2^31, up to the largest ensemble: ends, row ends and rows in the middle."""
+    n = R * (R - 1) // 2
+    assert rules.measure_tasks_(R) == R + n
+    assert _pair(rules, 0, R) == (0, 1) and _pair(rules, n - 1, R) == (R - 2, R - 1)
+    for r in (1, 2, R // 3, R // 2, R - 40, R - 3):
+        at = r * (2 * R - r - 1) // 2
+        assert _pair(rules, at, R) == (r, r + 1) and _pair(rules, at - 1, R) == (r - 1, R - 1)
