@@ -23,6 +23,7 @@ namespace {
 
 constexpr int kRowSmemMax = 227 * 1024;
 constexpr int kRowDraws = 32;  // updates whose random numbers are drawn at once, one lane each
+constexpr double kLeast = 4.9406564584124654e-324;  // the least positive double
 
 // Pair products in rows by p, the pair's distance from the middle of its sum: pair {x, s-x}, x < s-x, is the p-th of
 // sum s with p = (s-1)/2 - x.  Row p holds s = 2p+1 .. 2N-3-2p, so consecutive s (threads) are consecutive words, and
@@ -48,7 +49,7 @@ template <typename V> __device__ __forceinline__ V pair_product(V lo, V hi) {
 
 // A proposal as the rows use it.  test: FP32 the Metropolis uniform U; FP64 log U / (beta cc), drawn once with the proposal,
 // so that the decision is one comparison: dH = -cc share, and U < exp(-beta dH) is share > log U / (beta cc), which holds for
-// every dH <= 0 because log U < 0.
+// every dH <= 0 because log U < 0.  Where beta cc is infinite the quotient is -0; it is kept below zero, so that dH = 0 passes.
 template <typename real> struct RowProposal {
     typename vec2<real>::type aj, ak, nj, nk, dj, dk;
     real test;
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(MAXT, MINB) row_sweep_kernel(RowParams p) {
             pair_jk(p.seed, (uint32_t)si, (uint32_t)(base + sw), (uint32_t)u, N, j, k);
             pairs[at] = j | (k << 16);
             ProposalDraw<real> D = draw_proposal<real>(p.seed, cid, (uint32_t)(base + sw), (uint32_t)u);
-            if constexpr (sizeof(real) == 8) { D.pad = D.U; D.U = log(D.U) / (beta * cc); }
+            if constexpr (sizeof(real) == 8) { D.pad = D.U; D.U = fmin(log(D.U) / (beta * cc), -kLeast); }
             draws[at] = D;
         }
     };
