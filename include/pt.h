@@ -67,8 +67,10 @@ typedef struct pt_config {
     int measure_every;    /* sweeps between measurements; 0 = never */
     int resync_every;     /* sweeps between renormalisation + full FP64-accumulated H; 0 = never */
     int chains_per_block; /* chains sharing one J stream inside a thread block: 0 = tuned, or 8/16/32 */
-    int sweeps_per_unit;  /* sweeps in one scheduling unit of the persistent kernel; 0 = tuned */
-    int blocks_per_sm;    /* persistent thread blocks per SM; 0 = tuned */
+    int sweeps_per_unit;  /* sweeps in one scheduling unit of the persistent kernel; 0 = tuned.  Without effect on
+                           * ensembles that sweep one chain per block (see pt_default_shape) */
+    int blocks_per_sm;    /* persistent thread blocks per SM at most; 0 = tuned.  A limit keeps an ensemble on the
+                           * persistent kernel, as an explicit chains_per_block or consumer_warps does */
     int consumer_warps;   /* field-computing warps per thread block (plus one copy warp); 0 = tuned.  FP32:
                            * 7, 11 or 15 with 8 or 16 chains per block, 3, 7, 9 or 11 with 32; FP64: 7 with 8
                            * chains, 3 with 16 (PT_EINVAL otherwise) */
@@ -224,7 +226,7 @@ int pt_autotune(pt_ctx *ctx, int trial_sweeps, int *chosen);
  * Host-only, no device call: writes *chains_per_block (8, 16 or 32) and *consumer_warps.  The rule (measured on GB300):
  * 8 chains from N = 160 on; for 48 <= N < 160 the most chains per block (32 below N = 96, else 16, then 8) that still
  * give at least 0.8 x sm_count groups; 16 chains below N = 48; 8 when a sample has at most 8 chains; 11 field warps from
- * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block and consumer_warps 0, pt_create
+ * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block, consumer_warps and blocks_per_sm 0, pt_create
  * starts from it and departs where another kernel or shape measured faster: FP64 up to N = 160 and small FP32
  * ensembles up to N = 48 sweep one chain per block; FP32 ensembles of at most sm_count groups of 8 chains take 8 chains
  * per block, on clusters of blocks where an update has work for several; and below N = 48 it takes the most chains per

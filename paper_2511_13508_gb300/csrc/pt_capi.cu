@@ -1218,7 +1218,8 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     std::vector<SampleLayout> lay(S);
     std::vector<int> bo_all, xtlo_all, mode_all, ebo_all, eseg_all;
     std::vector<uint32_t> binfo_all;
-    if (!c->plain && !c->gfp32 && cfg.chains_per_block == 0 && cfg.consumer_warps == 0)
+    // a limit on the blocks per SM is one on the persistent blocks: it keeps them, as an explicit shape does
+    if (!c->plain && !c->gfp32 && cfg.chains_per_block == 0 && cfg.consumer_warps == 0 && cfg.blocks_per_sm == 0)
         c->row = row_path(c->dbl, c->maxN, (int64_t)S * chains_ps, sms);
     int64_t jblocks = 0, a_off = 0, q_off = 0, inc_total = 0, row_total = 0;
     int chain0 = 0;

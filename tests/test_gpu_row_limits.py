@@ -1,8 +1,10 @@
-"""One-chain-per-block sweeps (pt_row.cu) at the limits of their range: temperatures whose inverse is infinite."""
+"""One-chain-per-block sweeps (pt_row.cu) at the limits of their range: limits on the blocks per
+SM, which keep an ensemble on the J-sharing blocks, and temperatures whose inverse is infinite."""
 import numpy as np
 import pytest
 
 import paper_2511_13508_gb300 as pkg
+from paper_2511_13508_gb300 import workload
 
 pytestmark = pytest.mark.gpu
 
@@ -15,3 +17,17 @@ def test_zero_energy_change_is_accepted_at_infinite_beta(prec):
     p.sweep(5)
     o = p.observables()
     assert np.all(o["mc_att"] == 2 * 5 * 4) and np.array_equal(o["mc_acc"], o["mc_att"])
+
+
+@pytest.mark.parametrize("prec,N,G,w", [("fp64", 64, 16, 3), ("fp64", 128, 8, 7), ("fp32", 16, 16, 7)])
+def test_a_limit_on_the_blocks_keeps_the_block_kernel(prec, N, G, w):
+    """The kernels' energies differ by rounding, so equal bits mean the same kernel."""
+    Js = [workload.couplings(N, len(pkg.enumerate_quads(N)), 31)]
+    kw = dict(precision=prec, swap_every=4, measure_every=0, resync_every=0)
+    temps = workload.geometric_ladder(0.3, 1.6, 9)
+    runs = [pkg.PT([N], Js, temps, 2, 11, blocks_per_sm=1, **kw), pkg.PT([N], Js, temps, 2, 11, **kw),
+            pkg.PT([N], Js, temps, 2, 11, chains_per_block=G, consumer_warps=w, blocks_per_sm=1, **kw)]
+    for p in runs:
+        p.sweep(6)
+    E = [p.state()[1] for p in runs]
+    assert np.array_equal(E[0], E[2]) and not np.array_equal(E[1], E[2])
