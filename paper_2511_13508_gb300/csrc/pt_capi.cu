@@ -13,6 +13,7 @@
 #include <string>
 #include <thread>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/pt.h"
@@ -269,6 +270,18 @@ void *dev_alloc(pt_ctx *c, size_t bytes) {
     }
     if (p) c->allocs.push_back({p, bytes});
     return p;
+}
+
+// Gives a buffer of dev_alloc back before the context ends.
+template <typename T> void dev_free(pt_ctx *c, T *&p) {
+    for (size_t i = 0; p && i < c->allocs.size(); ++i)
+        if (c->allocs[i].first == p) {
+            if (c->free_) c->free_(p, c->user);
+            else cudaFree(p);
+            c->allocs.erase(c->allocs.begin() + i);
+            break;
+        }
+    p = nullptr;
 }
 
 template <typename T> int dalloc(pt_ctx *c, T **out, size_t count) {
@@ -1339,38 +1352,6 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
             for (int l = 0; l < c->N[s]; ++l) c->max_deg = std::max(c->max_deg, offs[s][l + 1] - offs[s][l]);
             hinc_off.insert(hinc_off.end(), offs[s].begin(), offs[s].end());
         }
-        if (c->gfp32 && graph_table_candidate(c->maxN, c->max_deg)) {
-            std::vector<GraphLists> lists(S);
-            auto make = [&](int s) {
-                const SampleDev &sd = c->samples[s];
-                graph_lists(c->N[s], sd.nq, graph + 4 * J_offsets[s], J + J_offsets[s], offs[s].data(), hrec.data() + sd.inc_off,
-                            hrecJ.data() + sd.inc_off, lists[s]);
-            };
-            if (!for_samples(S, 10 * q_off, make)) return bail(fail(c, PT_ENOMEM, "host allocation failed (graph lists)"));
-            int64_t nch = 0, ncr = 0, nco = 0, nxo = 0;
-            for (int s = 0; s < S; ++s) {
-                SampleDev &sd = c->samples[s];
-                sd.chunk_off = nch / 2; sd.cross_off = ncr; sd.xoff_off = nxo;
-                nch += (int64_t)lists[s].chunks.size(); ncr += (int64_t)lists[s].cross.size();
-                nco += (int64_t)lists[s].choff.size(); nxo += (int64_t)lists[s].xoff.size();
-                c->max_chunks = std::max(c->max_chunks, lists[s].max_chunks);
-                c->max_cross = std::max(c->max_cross, lists[s].max_cross);
-            }
-            // without room for them the sweep takes the incidence records
-            const bool room = dalloc(c, &c->d_chunks, nch) == PT_OK && dalloc(c, &c->d_cross, ncr) == PT_OK &&
-                              dalloc(c, &c->d_choff, nco) == PT_OK && dalloc(c, &c->d_xoff, nxo) == PT_OK;
-            if (!room) c->d_chunks = nullptr;
-            nco = 0;
-            for (int s = 0; room && s < S; ++s) {
-                const SampleDev &sd = c->samples[s];
-                const GraphLists &g = lists[s];
-                CK(cudaMemcpy(c->d_chunks + 2 * sd.chunk_off, g.chunks.data(), g.chunks.size() * sizeof(int4), cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c->d_cross + sd.cross_off, g.cross.data(), g.cross.size() * sizeof(int4), cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c->d_choff + nco, g.choff.data(), g.choff.size() * sizeof(int), cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c->d_xoff + sd.xoff_off, g.xoff.data(), g.xoff.size() * sizeof(int), cudaMemcpyHostToDevice));
-                nco += (int64_t)g.choff.size();
-            }
-        }
         RC(dalloc(c, &c->d_quads, hq.size()));
         RC(dalloc(c, &c->d_Jq, hJq.size()));
         RC(dalloc(c, &c->d_inc_off, hinc_off.size()));
@@ -1384,6 +1365,45 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
             RC(dalloc(c, &c->d_recJ, hrecJ.size()));
             CK(cudaMemcpy(c->d_rec, hrec.data(), hrec.size() * sizeof(int4), cudaMemcpyHostToDevice));
             CK(cudaMemcpy(c->d_recJ, hrecJ.data(), hrecJ.size() * sizeof(float), cudaMemcpyHostToDevice));
+        }
+        // Lists of the pair-table sweep: last, and all of them or none, since the sweep does without them (host or device memory
+        // short: the incidence records serve).
+        if (c->gfp32 && graph_table_candidate(c->maxN, c->max_deg)) {
+            std::vector<GraphLists> lists(S);
+            auto make = [&](int s) {
+                const SampleDev &sd = c->samples[s];
+                graph_lists(c->N[s], sd.nq, graph + 4 * J_offsets[s], J + J_offsets[s], offs[s].data(), hrec.data() + sd.inc_off,
+                            hrecJ.data() + sd.inc_off, lists[s]);
+            };
+            bool room = for_samples(S, 10 * q_off, make);
+            int64_t nch = 0, ncr = 0, nco = 0, nxo = 0;
+            for (int s = 0; room && s < S; ++s) {
+                SampleDev &sd = c->samples[s];
+                sd.chunk_off = nch / 2; sd.cross_off = ncr; sd.xoff_off = nxo;
+                nch += (int64_t)lists[s].chunks.size(); ncr += (int64_t)lists[s].cross.size();
+                nco += (int64_t)lists[s].choff.size(); nxo += (int64_t)lists[s].xoff.size();
+                c->max_chunks = std::max(c->max_chunks, lists[s].max_chunks);
+                c->max_cross = std::max(c->max_cross, lists[s].max_cross);
+            }
+            auto take = [&](auto **out, int64_t n) {
+                using T = std::remove_pointer_t<std::remove_pointer_t<decltype(out)>>;
+                if (room) *out = static_cast<T *>(dev_alloc(c, (size_t)n * sizeof(T)));
+                room = room && *out;
+            };
+            take(&c->d_chunks, nch); take(&c->d_cross, ncr); take(&c->d_choff, nco); take(&c->d_xoff, nxo);
+            if (!room) {
+                dev_free(c, c->d_chunks); dev_free(c, c->d_cross); dev_free(c, c->d_choff); dev_free(c, c->d_xoff);
+            }
+            nco = 0;
+            for (int s = 0; room && s < S; ++s) {
+                const SampleDev &sd = c->samples[s];
+                const GraphLists &g = lists[s];
+                CK(cudaMemcpy(c->d_chunks + 2 * sd.chunk_off, g.chunks.data(), g.chunks.size() * sizeof(int4), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_cross + sd.cross_off, g.cross.data(), g.cross.size() * sizeof(int4), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_choff + nco, g.choff.data(), g.choff.size() * sizeof(int), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(c->d_xoff + sd.xoff_off, g.xoff.data(), g.xoff.size() * sizeof(int), cudaMemcpyHostToDevice));
+                nco += (int64_t)g.choff.size();
+            }
         }
     }
     std::vector<int> label(c->n_chains), perm(c->n_chains);
