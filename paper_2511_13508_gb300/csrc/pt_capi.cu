@@ -1323,9 +1323,25 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         }
         CK(cudaMemcpy(c->d_J, hJ.data(), hJ.size(), cudaMemcpyHostToDevice));
     }
-    if (c->plain || c->gfp32 || c->row || c->maxN <= 64) {
-        std::vector<int4> hq((size_t)std::max<int64_t>(q_off, 1));
-        std::vector<double> hJq((size_t)std::max<int64_t>(q_off, 1));
+    // Quadruplet lists: kept on the device by the paths that read them; other contexts fill the row store from them, once
+    const bool keep_quads = c->plain || c->gfp32 || c->maxN <= 64;
+    std::vector<int4> hq;
+    std::vector<double> hJq;
+    auto list_quads = [&](int s, std::vector<int32_t> &abcd) {
+        const SampleDev &sd = c->samples[s];
+        abcd.resize((size_t)4 * std::max<int64_t>(sd.nq, 1));
+        int64_t cnt = sd.nq;
+        if (graph) std::copy(graph + 4 * J_offsets[s], graph + 4 * J_offsets[s + 1], abcd.begin());
+        else pt_enumerate_quads(c->N[s], abcd.data(), &cnt);
+        for (int64_t q = 0; q < cnt; ++q) {
+            hq[sd.q_off + q] = make_int4(abcd[4 * q], abcd[4 * q + 1], abcd[4 * q + 2], abcd[4 * q + 3]);
+            hJq[sd.q_off + q] = J[J_offsets[s] + q];
+        }
+    };
+    const size_t n_quads = (size_t)std::max<int64_t>(q_off, 1);
+    if (keep_quads) {
+        hq.resize(n_quads);
+        hJq.resize(n_quads);
         std::vector<int> hinc_off, hinc((size_t)std::max<int64_t>(inc_total, 1));
         std::vector<int4> hrec(c->gfp32 ? hinc.size() : 0);
         std::vector<float> hrecJ(c->gfp32 ? hinc.size() : 0);
@@ -1333,16 +1349,10 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         auto build = [&](int s) {
             const int n = c->N[s];
             const SampleDev &sd = c->samples[s];
-            std::vector<int32_t> abcd((size_t)4 * std::max<int64_t>(sd.nq, 1));
-            int64_t cnt = sd.nq;
-            if (graph) std::copy(graph + 4 * J_offsets[s], graph + 4 * J_offsets[s + 1], abcd.begin());
-            else pt_enumerate_quads(n, abcd.data(), &cnt);
-            for (int64_t q = 0; q < cnt; ++q) {
-                hq[sd.q_off + q] = make_int4(abcd[4 * q], abcd[4 * q + 1], abcd[4 * q + 2], abcd[4 * q + 3]);
-                hJq[sd.q_off + q] = J[J_offsets[s] + q];
-            }
+            std::vector<int32_t> abcd;
+            list_quads(s, abcd);
             offs[s].resize(n + 1);
-            incidence_lists(n, cnt, abcd.data(), offs[s].data(), hinc.data() + sd.inc_off);
+            incidence_lists(n, sd.nq, abcd.data(), offs[s].data(), hinc.data() + sd.inc_off);
             if (c->gfp32)
                 incidence_records(n, abcd.data(), J + J_offsets[s], offs[s].data(), hinc.data() + sd.inc_off,
                                   hrec.data() + sd.inc_off, hrecJ.data() + sd.inc_off);
@@ -1432,21 +1442,6 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
 
     if (c->gfp32) CK(graph_prepare(graph_params(c)));
-    if (c->row) {
-        c->d_Jrow = dev_alloc(c, (size_t)row_total * c->esize);
-        if (!c->d_Jrow) c->row = false;  // no room for the second store: the J-sharing blocks sweep
-    }
-    if (c->row) {
-        CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
-        CK(launch_row_pack(c->dbl, c->d_samples, S, c->d_quads, c->d_Jq, c->d_Jrow, c->stream));
-        std::vector<int> order(c->n_chains);
-        for (int i = 0; i < c->n_chains; ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(),
-                         [&](int x, int y) { return c->N[c->chain_sample[x]] > c->N[c->chain_sample[y]]; });
-        RC(dalloc(c, &c->d_order, c->n_chains));
-        CK(cudaMemcpy(c->d_order, order.data(), c->n_chains * sizeof(int), cudaMemcpyHostToDevice));
-        CK(row_prepare(c->dbl, c->maxN));
-    }
     // ---- persistent grid
     if (!c->plain && !c->gfp32) {
         int dev = 0, sms = 0;
@@ -1460,6 +1455,52 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         c->grid = std::max(1, std::min((int)c->groups.size(), most));
         c->sms = sms;
         RC(dalloc(c, &c->d_epart, c->max_groups * (size_t)kEnergyPartsMax * 32));
+    }
+
+    // ---- row store, last: without room for it, its chain order or the lists it is filled from, the J-sharing blocks sweep
+    if (c->row) {
+        int4 *quads = c->d_quads;
+        double *Jq = c->d_Jq;
+        c->d_Jrow = dev_alloc(c, (size_t)row_total * c->esize);
+        c->d_order = static_cast<int *>(dev_alloc(c, c->n_chains * sizeof(int)));
+        if (!keep_quads) {
+            quads = static_cast<int4 *>(dev_alloc(c, n_quads * sizeof(int4)));
+            Jq = static_cast<double *>(dev_alloc(c, n_quads * sizeof(double)));
+            auto list = [&](int s) {
+                std::vector<int32_t> abcd;
+                list_quads(s, abcd);
+            };
+            try {
+                hq.resize(n_quads);
+                hJq.resize(n_quads);
+                c->row = for_samples(S, q_off, list) && quads && Jq;
+            } catch (const std::bad_alloc &) {
+                c->row = false;
+            }
+        }
+        c->row = c->row && c->d_Jrow && c->d_order;
+        if (c->row) {
+            if (!keep_quads) {
+                CK(cudaMemcpy(quads, hq.data(), hq.size() * sizeof(int4), cudaMemcpyHostToDevice));
+                CK(cudaMemcpy(Jq, hJq.data(), hJq.size() * sizeof(double), cudaMemcpyHostToDevice));
+            }
+            std::vector<int> order(c->n_chains);
+            for (int i = 0; i < c->n_chains; ++i) order[i] = i;
+            std::stable_sort(order.begin(), order.end(),
+                             [&](int x, int y) { return c->N[c->chain_sample[x]] > c->N[c->chain_sample[y]]; });
+            CK(cudaMemcpy(c->d_order, order.data(), c->n_chains * sizeof(int), cudaMemcpyHostToDevice));
+            CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
+            CK(launch_row_pack(c->dbl, c->d_samples, S, quads, Jq, c->d_Jrow, c->stream));
+            CK(row_prepare(c->dbl, c->maxN));
+            CK(cudaStreamSynchronize(c->stream));
+        } else {
+            dev_free(c, c->d_Jrow);
+            dev_free(c, c->d_order);
+        }
+        if (!keep_quads) {
+            dev_free(c, quads);
+            dev_free(c, Jq);
+        }
     }
 
     // ---- initial chains (exact beta = 0 draws) and their energies

@@ -1,5 +1,5 @@
 """Creation with less device memory than the fastest kernels want.  What a context cannot do without is allocated first; the
-stores of the faster sweeps (pair-table lists of a graph) come last, are left out when they do not fit
+stores of the faster sweeps (pair-table lists of a graph, row store of the comb) come last, are left out when they do not fit
 and are then given back whole, so that whatever fits without them is created and runs on the other kernels.
 
 The allocator callbacks count bytes and refuse what passes a limit; no allocation of the device fails.
@@ -86,3 +86,23 @@ def test_graph_lists_give_way(create):
     p, held = create(least, *args, **kw)
     assert p is not None and held == least
     assert create(least - 256, *args, **kw)[0] is None
+
+
+@pytest.mark.parametrize("prec,N,G", [("fp64", 66, 16), ("fp64", 24, 16), ("fp64", 160, 8), ("fp32", 24, 16)])
+def test_row_store_gives_way(create, prec, N, G):
+    Js = [workload.couplings(N, len(pkg.enumerate_quads(N)), 5)]
+    args = ([N], Js, workload.geometric_ladder(0.3, 1.6, 5), 2, 17)
+    kw = dict(precision=prec, swap_every=2, measure_every=2, resync_every=0)
+    block, base = create(ALL, *args, **dict(kw, chains_per_block=G))
+    full, need = create(ALL, *args, **kw)
+    # beside what the J-sharing blocks hold, a context keeps the row store and the order of its chains
+    row = N * (N // 2) * N * (8 if prec == "fp64" else 4)
+    assert base + row <= need <= base + row + 1024, (need - base, row)
+    for lack in (256, row // 2, row):
+        p, held = create(need - lack, *args, **kw)
+        assert p is not None and held == base, (lack, held, base)
+        same_run(p, block if lack == 256 else create(ALL, *args, **dict(kw, chains_per_block=G))[0], 3, 1e-12 if prec == "fp64" else 1e-5)
+    p, held = create(base, *args, **kw)
+    assert p is not None and held == base
+    assert create(base - 256, *args, **kw)[0] is None
+    same_run(full, create(ALL, *args, **kw)[0], 3, 0.0)
