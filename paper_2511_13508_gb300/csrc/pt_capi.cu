@@ -21,6 +21,7 @@
 #include "pt_gemm.h"
 #include "pt_kernels.h"
 #include "pt_learn.h"
+#include "pt_rules.h"
 
 using namespace ptgb;
 
@@ -235,7 +236,7 @@ struct pt_ctx {
     bool own_stream = false;
     size_t max_groups = 0;  // capacity of d_groups / d_progress (groups of 8 chains)
     int sms = 0;            // streaming multiprocessors of the device
-    double *d_epart = nullptr;  // partial energies of the resync, [max_groups][kEnergyPartsMax][32]
+    double *d_epart = nullptr;  // partial energies of the resync, [group][part][32]
     LearnState *learn = nullptr;
     unsigned long long *d_gm_acc = nullptr, *d_gm_att = nullptr;  // [S][nT] global-move counters
 };
@@ -398,19 +399,9 @@ int run_energy(pt_ctx *c, int renorm, double *E_out, bool write_state) {
     p.samples = c->d_samples; p.groups = c->d_groups; p.J = c->d_J; p.bo = c->d_bo; p.blkinfo = c->d_blkinfo;
     p.mode_blk = c->d_mode_blk; p.ebo = c->d_ebo; p.a = c->d_a; p.cc = c->cfg.cc_factor; p.renorm = renorm;
     p.E_out = E_out; p.E_state = write_state ? c->d_E : nullptr; p.ctl = c->d_ctl;
-    // several thread blocks per group, their partial sums added in a fixed order by a second kernel.  FP64: about 8 blocks
-    // per SM (it waits on coupling loads).  FP32: one block per SM at a time, so the number of parts that leaves the least
-    // of the last wave idle, each part counted with the 2% that loading the group's tables takes
-    const int ng = (int)c->groups.size(), sms = std::max(c->sms, 1);
+    const int ng = (int)c->groups.size();
     p.part = c->d_epart; p.eseg = c->d_eseg; p.maxN = c->maxN;
-    if (c->dbl) p.parts = std::max(1, std::min(8, (8 * sms + ng - 1) / std::max(ng, 1)));
-    else {
-        double best = 1e30;
-        for (int q = 1; q <= kEnergyPartsMax; ++q) {
-            const double t = (double)((ng * q + sms - 1) / sms) / q * (1.0 + 0.02 * q);
-            if (t < best) { best = t; p.parts = q; }
-        }
-    }
+    p.parts = energy_parts(c->dbl, ng, std::max(c->sms, 1));
     const int Ge = c->dbl ? std::min(c->G, 16) : c->G;
     CK(launch_energy(c->dbl, Ge, p, ng, c->maxN, c->stream));
     return PT_OK;
@@ -1454,7 +1445,12 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         c->most = most;
         c->grid = std::max(1, std::min((int)c->groups.size(), most));
         c->sms = sms;
-        RC(dalloc(c, &c->d_epart, c->max_groups * (size_t)kEnergyPartsMax * 32));
+        size_t parts = 0;  // of every grouping a shape of this context can make
+        for (int g : {8, 16, 32}) {
+            const int ng = S * ((chains_ps + g - 1) / g);
+            parts = std::max(parts, (size_t)ng * energy_parts(c->dbl, ng, std::max(sms, 1)));
+        }
+        RC(dalloc(c, &c->d_epart, parts * 32));
     }
 
     // ---- row store, last: without room for it, its chain order or the lists it is filled from, the J-sharing blocks sweep

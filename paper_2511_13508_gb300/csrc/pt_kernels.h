@@ -67,12 +67,11 @@ struct EnergyParams {
     double *E_out;   // optional: energies by chain slot
     double *E_state; // optional: running-energy array to overwrite
     Control *ctl;
-    double *part;    // partial sums [group][part][32] (kEnergyPartsMax parts at most)
-    int parts;       // thread blocks per group (1 .. kEnergyPartsMax)
+    double *part;    // partial sums [group][part][32]
+    int parts;       // thread blocks per group (energy_parts)
     const int *eseg; // FP32, per sample: prefix count over the tiles (blocks) of their runs of modes (nblk+1, at seg_off)
     int maxN;
 };
-constexpr int kEnergyPartsMax = 16;
 constexpr int kEnergySeg = 64;  // modes of a run
 // pt_energy.cu: the partial sums of FP32 chains
 cudaError_t launch_energy_tiles(int G, const EnergyParams &p, int ngroups, cudaStream_t s);

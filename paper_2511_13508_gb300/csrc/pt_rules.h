@@ -1,6 +1,7 @@
 // pt_rules.h -- index and scheduling arithmetic of the kernels and their launchers, free of CUDA so that a host compiler
 // takes it too (tests/test_rules_host.py runs it at sizes no GPU test reaches).
 #pragma once
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -36,6 +37,21 @@ PT_HD inline void replica_pair(int64_t at, int R, int *r1, int *r2) {
     while (row(r + 1) <= at) ++r;
     *r1 = (int)r;
     *r2 = (int)(r + 1 + (at - row(r)));
+}
+
+// Thread blocks a group's full energy is split over, their partial sums added in a fixed order by a second kernel.  FP64: about
+// 8 blocks per SM (it waits on coupling loads).  FP32: one block per SM at a time, so the number of parts that leaves the least
+// of the last wave idle, each part counted with the 2% that loading the group's tables takes.
+constexpr int kEnergyPartsMax = 16;
+inline int energy_parts(bool fp64, int groups, int sms) {
+    if (fp64) return std::max(1, std::min(8, (8 * sms + groups - 1) / std::max(groups, 1)));
+    double best = 1e30;
+    int parts = 1;
+    for (int q = 1; q <= kEnergyPartsMax; ++q) {
+        const double t = (double)(((int64_t)groups * q + sms - 1) / sms) / q * (1.0 + 0.02 * q);
+        if (t < best) { best = t; parts = q; }
+    }
+    return parts;
 }
 
 }  // namespace ptgb

@@ -17,6 +17,7 @@
 #include "pt_bulk.cuh"
 #include "pt_common.cuh"
 #include "pt_kernels.h"
+#include "pt_rules.h"
 #include "pt_move.cuh"
 
 namespace ptgb {

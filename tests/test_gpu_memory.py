@@ -106,3 +106,13 @@ def test_row_store_gives_way(create, prec, N, G):
     assert p is not None and held == base
     assert create(base - 256, *args, **kw)[0] is None
     same_run(full, create(ALL, *args, **kw)[0], 3, 0.0)
+
+
+def test_partial_energies_follow_the_groups(create):
+    """Partial sums of the full energy take 256 bytes per group and part; an FP64 ensemble of 1024 groups of 8 has two parts, and
+    the state, its snapshot and the books of a chain of 4 modes stay below 330 bytes."""
+    Js = [workload.couplings(4, 1, 5)]
+    p, held = create(ALL, [4], Js, [0.5, 1.0], 4096, 17, precision="fp64", chains_per_block=8, swap_every=0, measure_every=0)
+    assert held <= 8192 * (330 + 64), held / 8192
+    p.resync()
+    assert np.isfinite(p.energy()).all()
