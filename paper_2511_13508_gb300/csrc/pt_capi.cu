@@ -1888,11 +1888,13 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
     Cand bestc = {c->row ? 0 : c->G, c->row ? 0 : c->ncw, c->spu};
+    const int G0 = c->G, ncw0 = c->ncw;
     auto set = [&](const Cand &cd) {
         if (cd.G > 0) return set_shape(c, cd.G, cd.ncw, cd.spu);
-        c->row = true;
-        drop_graphs(c);
-        return (int)PT_OK;
+        // one chain per block: full energies still run on the context's groups, which other trials have replaced
+        const int rc = set_shape(c, G0, ncw0, cd.spu);
+        if (rc == PT_OK) c->row = true;
+        return rc;
     };
     for (const Cand &cd : cands) {
         if (set(cd) != PT_OK) continue;
