@@ -218,7 +218,9 @@ int pt_load(pt_ctx *ctx, const void *buf, size_t len);
  * every supported shape for trial_sweeps sweeps on the live ensemble, keeps the fastest and restores
  * the ensemble (state, counters, accumulators) exactly as before the call.  chosen (optional, 3 ints)
  * receives {chains_per_block, consumer_warps, sweeps_per_unit}, {0, 0, sweeps_per_unit} when one chain per block (which
- * pt_create takes by itself for those ensembles) is the fastest.  PT_EUNSUPPORTED for the plain path. */
+ * pt_create takes by itself for those ensembles) is the fastest.  FP32 contexts with pt_config.sweeps_per_unit = 0 cut the work
+ * of each launch themselves: their unit is not tuned, the third value is the default unit, and a new context takes the schedule
+ * that was timed with sweeps_per_unit = 0.  PT_EUNSUPPORTED for the plain path. */
 int pt_autotune(pt_ctx *ctx, int trial_sweeps, int *chosen);
 
 /* The sweep-block shape of a batch by size alone: of n_samples samples whose largest mode count is max_n (even,

@@ -329,7 +329,8 @@ class PT:
 
     def autotune(self, trial_sweeps=8):
         """Times the supported sweep-block shapes on the live ensemble, keeps the fastest and restores
-        the ensemble; returns (chains_per_block, consumer_warps, sweeps_per_unit)."""
+        the ensemble; returns (chains_per_block, consumer_warps, sweeps_per_unit), the first two 0 for one chain per block.
+        FP32 with sweeps_per_unit=0: the third is the default unit, unused (pass 0 for the schedule timed)."""
         out = (ctypes.c_int * 3)()
         self._c(lib().pt_autotune(self._h, int(trial_sweeps), out))
         return tuple(out)

@@ -1875,13 +1875,15 @@ int pt_autotune(pt_ctx *c, int trial_sweeps, int *chosen) {
     struct Cand { int G, ncw, spu; };
     std::vector<Cand> cands;
     if (c->d_Jrow) cands.push_back({0, 0, spu0});  // one chain per block
+    const bool own_runs = !c->dbl && c->cfg.sweeps_per_unit == 0;  // launches that cut their runs themselves use no unit
     const int Gs_f[] = {8, 16, 32}, Gs_d[] = {8, 16};
     const int ncws[] = {3, 7, 9, 11, 15};
     for (int G : (c->dbl ? std::vector<int>(Gs_d, Gs_d + 2) : std::vector<int>(Gs_f, Gs_f + 3))) {
         if (G > 8 && cps < G / 2) continue;  // mostly empty blocks
         for (int n : ncws)
             if (shape_exists(c->dbl, G, n))
-                for (int sp : {spu0, spu0 * 4}) cands.push_back({G, n, sp});
+                for (int sp : {spu0, spu0 * 4})
+                    if (sp == spu0 || !own_runs) cands.push_back({G, n, sp});
     }
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));

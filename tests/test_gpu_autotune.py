@@ -1,4 +1,4 @@
-"""pt_autotune on ensembles that one chain per block serves best."""
+"""pt_autotune on ensembles that one chain per block serves best, and what it says about the units of a launch."""
 import numpy as np
 import pytest
 
@@ -18,3 +18,14 @@ def test_one_chain_per_block_leaves_the_groups_alone(prec, N, nT):
     E = p.energy()
     assert p.autotune(4)[:2] == (0, 0)
     assert np.array_equal(p.energy(), E)
+
+
+def test_units_are_the_default_where_the_launch_cuts_its_own():
+    """FP32 without an explicit unit: each launch cuts its runs itself, the tuner reports the default unit (8 sweeps from
+    N = 48 on), whatever was timed; an explicit unit is tuned."""
+    N = 64
+    Js = [workload.couplings(N, len(pkg.enumerate_quads(N)), 3)]
+    p = pkg.PT([N], Js, workload.geometric_ladder(0.3, 1.6, 16), 2, 3, swap_every=16, measure_every=4, resync_every=32)
+    assert {p.autotune(2)[2] for _ in range(6)} == {8}
+    q = pkg.PT([N], Js, workload.geometric_ladder(0.3, 1.6, 16), 2, 3, sweeps_per_unit=2)
+    assert q.autotune(2)[2] in (2, 8)
