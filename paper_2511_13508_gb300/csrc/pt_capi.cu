@@ -337,23 +337,6 @@ bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
     return maxN <= 48 && n_chains <= (maxN <= 32 ? 6 : 2) * (int64_t)sms;
 }
 
-// Runs each group's updates are cut into on a device that holds `most` groups at once: those that leave the least of the last
-// round of units idle.  A unit costs about 8 us beside its updates (tables, amplitudes, the first couplings), an update of
-// the largest N about 2 + N^2 / 6000 us (GB300).  Measured there against one run per group and sweep (192 groups of
-// N = 256 on 152 SMs): 2298 -> 2127 us per sweep at 8 sweeps a launch, where the second round left 112 SMs idle.
-int sweep_runs(int groups, int most, int64_t updates, int maxN) {
-    const double group_us = (double)updates * (2.0 + maxN * (double)maxN / 6000.0);
-    const int top = (int)std::max<int64_t>(1, std::min<int64_t>(updates, 512));
-    int best = 1;
-    double best_t = 1e300;
-    for (int k = 1; k <= top; ++k) {
-        const int64_t rounds = std::max<int64_t>(k, ((int64_t)groups * k + most - 1) / std::max(most, 1));  // runs of a group queue up
-        const double t = (double)rounds * (group_us / k + 8.0);
-        if (t < best_t) { best_t = t; best = k; }
-    }
-    return best;
-}
-
 // Blocks per group of the FP32 sweep (a cluster) when its groups leave SMs idle: the most that keep all groups resident
 // at once, and no more than an update has chunks for.  Measured on GB300 (us per sweep of one sample, 8 chains x 7
 // warps, 1 / 2 / 4 / 8 blocks): N = 256, 12 groups 1680 / 1057 / 633 / 428; N = 160, 8 groups 509 / 349 / 247 / 180;
@@ -464,7 +447,7 @@ int run_sweeps(pt_ctx *c, int seg) {
     p.bo = c->d_bo; p.xtlo = c->d_xtlo; p.blkinfo = c->d_blkinfo; p.mode_blk = c->d_mode_blk; p.a = c->d_a;
     p.E = c->d_E; p.label = c->d_label; p.beta = c->d_beta; p.mc_acc = c->d_mc_acc; p.mc_att = c->d_mc_att;
     p.R = c->R; p.nT = c->nT; p.maxN = c->maxN; p.seed = c->seed; p.cc = c->cfg.cc_factor; p.ctl = c->d_ctl;
-    p.progress = c->d_progress; p.n_sweeps = seg; p.sweeps_per_unit = std::min(c->spu, seg);
+    p.progress = c->d_progress; p.n_sweeps = seg; p.sweeps_per_unit = unit_sweeps(seg, c->spu, (int)c->groups.size());
     p.measure_every = c->cfg.measure_every; p.snap_a = c->d_snap_a; p.snap_E = c->d_snap_E;
     p.n_snap_max = c->n_snap_max; p.a_total = c->a_total; p.n_chains = c->n_chains; p.trace = c->d_trace;
     p.runs = (seg + p.sweeps_per_unit - 1) / p.sweeps_per_unit;

@@ -14,6 +14,8 @@ extern "C" {
 int64_t grid_warp_(unsigned b, unsigned n, unsigned t) { return grid_warp(b, n, t); }
 int64_t measure_tasks_(int R) { return measure_tasks(R); }
 void replica_pair_(int64_t at, int R, int *r1, int *r2) { replica_pair(at, R, r1, r2); }
+int unit_sweeps_(int seg, int sweeps, int groups) { return unit_sweeps(seg, sweeps, groups); }
+int sweep_runs_(int groups, int most, int64_t updates, int maxN) { return sweep_runs(groups, most, updates, maxN); }
 }
 """
 
@@ -27,6 +29,7 @@ def rules(tmp_path_factory):
                     str(d / "shim.cpp"), "-o", so], check=True)
     L = ctypes.CDLL(so)
     L.grid_warp_.restype = L.measure_tasks_.restype = ctypes.c_int64
+    L.sweep_runs_.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int64, ctypes.c_int]
     L.replica_pair_.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
     return L
 
@@ -60,3 +63,23 @@ def test_replica_pairs_of_very_many_replicas(rules, R):
     for r in (1, 2, R // 3, R // 2, R - 40, R - 3):
         at = r * (2 * R - r - 1) // 2
         assert _pair(rules, at, R) == (r, r + 1) and _pair(rules, at - 1, R) == (r - 1, R - 1)
+
+
+@pytest.mark.parametrize("seg,sweeps,groups", [(64, 1, 192), (64, 8, 1), (7, 32, 5000), (1 << 20, 1, 5000), (1 << 28, 1, 12),
+                                               (1 << 29, 3, 1), (64, 1, 1 << 25), (1 << 20, 1, 1 << 25)])
+def test_units_of_a_launch_fit_32_bits(rules, seg, sweeps, groups):
+    unit = rules.unit_sweeps_(seg, sweeps, groups)
+    assert 1 <= unit <= seg and unit >= min(seg, sweeps)
+    units = -(-seg // unit) * groups
+    assert units <= 1 << 30
+    if -(-seg // sweeps) * groups <= 1 << 30:
+        assert unit == min(seg, sweeps)
+
+
+@pytest.mark.parametrize("groups", [1, 152, 160, 192, 5000, 1 << 20, 3 << 20, 1 << 23, 1 << 25])
+@pytest.mark.parametrize("updates,N", [(2, 4), (224, 64), (8192, 256), (1 << 30, 64)])
+def test_runs_of_a_launch_fit_32_bits(rules, groups, updates, N):
+    runs = rules.sweep_runs_(groups, 152, updates, N)
+    assert 1 <= runs <= updates and runs * groups <= 1 << 30
+    if groups <= 152:
+        assert runs == 1
