@@ -231,8 +231,8 @@ int pt_autotune(pt_ctx *ctx, int trial_sweeps, int *chosen);
  * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block, consumer_warps and blocks_per_sm 0, pt_create
  * starts from it and departs where another kernel or shape measured faster: FP64 up to N = 160 and small FP32
  * ensembles up to N = 48 sweep one chain per block; FP32 ensembles of at most sm_count groups of 8 chains take 8 chains
- * per block, on clusters of blocks where an update has work for several; and below N = 48 it takes the most chains per
- * block that fill the device.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL otherwise, and for out-of-range
+ * per block, on clusters of blocks where an update has work for several; and larger ones below N = 48 take 32 chains per
+ * block where that gives at least 0.8 x sm_count groups.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL otherwise, and for out-of-range
  * arguments or NULL outputs). */
 int pt_default_shape(int precision, int max_n, int n_samples, int chains_per_sample, int sm_count,
                      int *chains_per_block, int *consumer_warps);

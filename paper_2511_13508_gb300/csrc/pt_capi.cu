@@ -1039,8 +1039,11 @@ static void default_shape(bool dbl, int maxN, int S, int chains_ps, int sms, int
 // - an ensemble of no more groups of 8 than SMs gives each of them a block, or a cluster of blocks of 7 warps (a block's
 //   update takes as long for 8 chains as for 32 when it is alone on its SM: N = 64, 168 chains 78 us per sweep with 8
 //   chains a block, 71 on clusters of 4, 162 with 32 chains);
-// - below N = 48 it takes the most chains per block that still fill the SMs (N = 32, 4096 chains: 39.6 us with 32
-//   chains x 7 warps, 64.7 with 16 x 7; N = 16: 13.2, 28.1).
+// - below N = 48 it takes 32 chains per block where those still fill the SMs (N = 32, 4096 chains: 39.6 us with 32
+//   chains x 7 warps, 64.7 with 16 x 7; N = 16: 13.2, 28.1).  Between the two stay 16: groups of 8 that do not all fit at
+//   once take a second round (64 sweeps, N = 16, 1280 / 1600 / 1888 chains: 16 x 7 892 / 970 / 975 us, 8 x 7 1064 / 1263 /
+//   1538; N = 32 2124 / 2229 / 2228, 2124 / 2536 / 3051; N = 46 3780 / 3976 / 4040, 3256 / 4043 / 4897, where single sweeps
+//   at 1280 chains take 75 and 91).
 static void tuned_shape(int maxN, int S, int chains_ps, int sms, int *G, int *ncw) {
     if (sms < 1) return;
     const int64_t g8 = (int64_t)S * ((chains_ps + 7) / 8);
@@ -1049,11 +1052,7 @@ static void tuned_shape(int maxN, int S, int chains_ps, int sms, int *G, int *nc
         *ncw = maxN < 48 || cluster_blocks(8, 7, maxN, (int)g8, sms) > (maxN >= 160 ? 2 : 1) ? 7 : 11;
         return;
     }
-    if (maxN >= 48) return;
-    *G = 8;
-    for (int g : {32, 16})
-        if (*G == 8 && chains_ps > g / 2 && (int64_t)S * ((chains_ps + g - 1) / g) >= (int64_t)sms * 4 / 5) *G = g;
-    *ncw = 7;
+    if (maxN < 48 && chains_ps > 16 && (int64_t)S * ((chains_ps + 31) / 32) >= (int64_t)sms * 4 / 5) *G = 32;
 }
 
 int pt_default_shape(int precision, int max_n, int n_samples, int chains_per_sample, int sm_count,
