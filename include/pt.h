@@ -228,12 +228,13 @@ int pt_autotune(pt_ctx *ctx, int trial_sweeps, int *chosen);
  * Host-only, no device call: writes *chains_per_block (8, 16 or 32) and *consumer_warps.  The rule (measured on GB300):
  * 8 chains from N = 160 on; for 48 <= N < 160 the most chains per block (32 below N = 96, else 16, then 8) that still
  * give at least 0.8 x sm_count groups; 16 chains below N = 48; 8 when a sample has at most 8 chains; 11 field warps from
- * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block, consumer_warps and blocks_per_sm 0, pt_create
- * starts from it and departs where another kernel or shape measured faster: FP64 up to N = 160 and small FP32
- * ensembles up to N = 48 sweep one chain per block; FP32 ensembles of at most sm_count groups of 8 chains take 8 chains
- * per block, on clusters of blocks where an update has work for several; and larger ones below N = 48 take 32 chains per
- * block where that gives at least 0.8 x sm_count groups.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL otherwise, and for out-of-range
- * arguments or NULL outputs). */
+ * N = 48 on, else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3.  With chains_per_block, consumer_warps and
+ * blocks_per_sm 0, pt_create starts from it and departs where another kernel or shape measured faster: FP64 up to
+ * N = 160 (but for large ensembles of N = 4) and small FP32 ensembles up to N = 48 sweep one chain per block; FP32
+ * ensembles of at most sm_count groups of 8 chains take 8 chains per block, on clusters of blocks where an update has
+ * work for several; and larger ones below N = 48 take 32 chains per block where that gives at least 0.8 x sm_count
+ * groups.  precision: PT_PREC_FP32 or PT_PREC_FP64 (PT_EINVAL otherwise, and for out-of-range arguments or NULL
+ * outputs). */
 int pt_default_shape(int precision, int max_n, int n_samples, int chains_per_sample, int sm_count,
                      int *chains_per_block, int *consumer_warps);
 

@@ -326,14 +326,17 @@ int watchdog_sync(pt_ctx *c) {
 
 // ---------------------------------------------------------------------------------- kernels
 // Whether a comb context of default shape sweeps on the one-chain-per-block kernel.
-// FP64: wherever its pair products fit in shared memory.  It was the faster one at every size measured on GB300 (us per
-// sweep against 16 x 3 / 8 x 7 blocks): N = 16, 64 chains 16.7 | 268 / 309; N = 64, 1024 chains 856 | 4187 / 2230, 4096
-// chains 3460 | 6110 / 8690; N = 128, 512 chains 2990 | 24500 / 10270.
+// FP64: wherever its pair products fit in shared memory.  Measured on GB300 (us per sweep against 16 x 3 / 8 x 7 blocks):
+// N = 16, 64 chains 16.7 | 268 / 309; N = 64, 1024 chains 856 | 4187 / 2230, 4096 chains 3460 | 6110 / 8690; N = 128, 512
+// chains 2990 | 24500 / 10270.  A launch draws random numbers a warp at a time for each chain, which a launch of few updates
+// pays for in full: at N = 4 (2 updates a sweep), with more than 16 chains per SM, the blocks of 16 chains keep the sweep
+// (launches of 1 / 8 sweeps, own block | 16 x 3, 4096 chains 88 / 347 | 66 / 432, 65536 chains 1228 / 5172 | 769 / 5716); at N = 6
+// and 8 only launches of single sweeps of 65536 chains are slower, by 7 and 9%, and those of 8 sweeps faster by 34 and 27%.
 // FP32: as long as few chains share an SM, since a block then waits on latencies that sharing couplings does not
 // shorten (168 chains, against the best block shape: N = 16 5.2 | 13.4, N = 32 14.3 | 32, N = 48 40 | 56, N = 64 69 | 70;
 // 1024 chains: N = 16 7.9 | 13.2, N = 32 30 | 34, N = 40 51 | 43; 4096 chains: N = 16 27 | 13.7).
 bool row_path(bool dbl, int maxN, int64_t n_chains, int sms) {
-    if (dbl) return maxN <= 160;
+    if (dbl) return maxN <= 160 && (maxN > 4 || n_chains <= 16 * (int64_t)sms);
     return maxN <= 48 && n_chains <= (maxN <= 32 ? 6 : 2) * (int64_t)sms;
 }
 

@@ -1,5 +1,5 @@
 """One-chain-per-block sweeps (pt_row.cu) at the limits of their range: limits on the blocks per
-SM, which keep an ensemble on the J-sharing blocks, and temperatures whose inverse is infinite."""
+SM, which keep an ensemble on the J-sharing blocks, the smallest N, and temperatures whose inverse is infinite."""
 import numpy as np
 import pytest
 
@@ -31,3 +31,19 @@ def test_a_limit_on_the_blocks_keeps_the_block_kernel(prec, N, G, w):
         p.sweep(6)
     E = [p.state()[1] for p in runs]
     assert np.array_equal(E[0], E[2]) and not np.array_equal(E[1], E[2])
+
+
+def test_small_fp64_launches():
+    """N = 4: with more than 16 chains per SM the J-sharing blocks sweep, with fewer a block per chain does."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    Js = [workload.couplings(4, len(pkg.enumerate_quads(4)), 31)]
+    kw = dict(precision="fp64", swap_every=4, measure_every=0, resync_every=0)
+    for R, row in ((sms // 2, True), (2 * sms + 1, False)):  # 8 temperatures
+        temps = workload.geometric_ladder(0.3, 1.6, 8)
+        a, b = pkg.PT([4], Js, temps, R, 11, **kw), pkg.PT([4], Js, temps, R, 11, chains_per_block=16, **kw)
+        for p in (a, b):
+            p.sweep(30)
+        (x, E), (y, F) = a.state(), b.state()
+        assert np.abs(x - y).max() <= 1e-13 and np.abs(E - F).max() <= 1e-11
+        assert np.array_equal(E, F) != row
