@@ -221,6 +221,7 @@ struct pt_ctx {
     Control *d_ctl = nullptr;
     void *d_snap_a = nullptr;
     double *d_snap_E = nullptr;
+    size_t snap_bytes = 0;  // of d_snap_a
     int n_snap_max = 0, max_seg = 0;
     int4 *d_quads = nullptr;
     int4 *d_rec = nullptr;     // incidence records of the FP32 quadruplet-list path
@@ -1259,7 +1260,8 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     RC(dalloc(c, &c->d_eseg, eseg_all.size()));
     c->d_a = dev_alloc(c, (size_t)c->a_total * 2 * c->esize);
     if (!c->d_a) return bail(fail(c, PT_ENOMEM, "device allocation failed (state)"));
-    c->d_snap_a = dev_alloc(c, (size_t)c->n_snap_max * c->a_total * 2 * c->esize);
+    c->snap_bytes = snapshot_bytes(c->n_snap_max, c->a_total, c->esize);
+    c->d_snap_a = dev_alloc(c, c->snap_bytes);
     if (!c->d_snap_a) return bail(fail(c, PT_ENOMEM, "device allocation failed (snapshots)"));
     RC(dalloc(c, &c->d_snap_E, (size_t)c->n_snap_max * c->n_chains));
     RC(dalloc(c, &c->d_E, c->n_chains));
@@ -1633,8 +1635,8 @@ int pt_get_state(pt_ctx *c, double *a, double *E) {
     if (!c) return fail(nullptr, PT_EINVAL, "pt_get_state: NULL context");
     // Amplitudes (widened to FP64) and energies are put in canonical order on the device, so that each is a plain copy.
     // The snapshots, which hold nothing between segments, serve as the buffer: the state goes through in as many pieces
-    // as that takes (one with two FP32 snapshots or an FP64 one, else two).
-    const int64_t cap = std::max<int64_t>(1, (int64_t)((size_t)c->n_snap_max * c->a_total * 2 * c->esize / sizeof(double2)));
+    // as that takes (one with two FP32 snapshots or an FP64 one, or up to 1 MB, else two).
+    const int64_t cap = (int64_t)(c->snap_bytes / sizeof(double2));
     double2 *canon = reinterpret_cast<double2 *>(c->d_snap_a);
     for (int64_t lo = 0; lo == 0 || (a && lo < c->a_total); lo += cap) {
         const int64_t n = std::min(cap, c->a_total - lo);

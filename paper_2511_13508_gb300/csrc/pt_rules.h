@@ -3,6 +3,7 @@
 #pragma once
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 
 #ifdef __CUDACC__
@@ -78,6 +79,14 @@ inline int sweep_runs(int groups, int most, int64_t updates, int maxN) {
         if (t < best_t) { best_t = t; best = k; }
     }
     return best;
+}
+
+// Bytes of the snapshot buffer: n_snap states of the chains (pairs of reals).  A host readout passes through it widened to FP64, in
+// as many pieces as that takes; FP32 with one snapshot would need two, which costs a small state more than the copy itself
+// (N = 64, 12 chains: 72 us against 46 in one piece; N = 256, 96 chains: 98 against 65, on GB300), so up to 1 MB it has the room.
+inline size_t snapshot_bytes(int n_snap, int64_t a_total, size_t real_bytes) {
+    const size_t wide = (size_t)a_total * 16;
+    return std::max((size_t)n_snap * (size_t)a_total * 2 * real_bytes, std::min(wide, (size_t)1 << 20));
 }
 
 }  // namespace ptgb

@@ -16,6 +16,7 @@ int64_t measure_tasks_(int R) { return measure_tasks(R); }
 void replica_pair_(int64_t at, int R, int *r1, int *r2) { replica_pair(at, R, r1, r2); }
 int unit_sweeps_(int seg, int sweeps, int groups) { return unit_sweeps(seg, sweeps, groups); }
 int sweep_runs_(int groups, int most, int64_t updates, int maxN) { return sweep_runs(groups, most, updates, maxN); }
+int64_t snapshot_bytes_(int n, int64_t a, int real) { return (int64_t)snapshot_bytes(n, a, (size_t)real); }
 }
 """
 
@@ -29,6 +30,7 @@ def rules(tmp_path_factory):
                     str(d / "shim.cpp"), "-o", so], check=True)
     L = ctypes.CDLL(so)
     L.grid_warp_.restype = L.measure_tasks_.restype = ctypes.c_int64
+    L.snapshot_bytes_.argtypes, L.snapshot_bytes_.restype = [ctypes.c_int, ctypes.c_int64, ctypes.c_int], ctypes.c_int64
     L.sweep_runs_.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int64, ctypes.c_int]
     L.replica_pair_.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]
     return L
@@ -83,3 +85,11 @@ def test_runs_of_a_launch_fit_32_bits(rules, groups, updates, N):
     assert 1 <= runs <= updates and runs * groups <= 1 << 30
     if groups <= 152:
         assert runs == 1
+
+
+@pytest.mark.parametrize("n,a,real,pieces", [(1, 2, 4, 1), (1, 768, 4, 1), (1, 65536, 4, 1), (1, 65538, 4, 2), (1, 1 << 30, 4, 2),
+                                             (2, 1 << 30, 4, 1), (5, 18, 4, 1), (1, 16, 8, 1), (1, 1 << 30, 8, 1)])
+def test_snapshots_hold_a_readout(rules, n, a, real, pieces):
+    """A state of a FP64 pairs passes through the snapshot buffer in this many pieces."""
+    room = rules.snapshot_bytes_(n, a, real)
+    assert room >= n * a * 2 * real and -(-a // (room // 16)) == pieces
