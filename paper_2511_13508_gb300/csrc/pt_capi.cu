@@ -388,8 +388,9 @@ int run_energy(pt_ctx *c, int renorm, double *E_out, bool write_state) {
     p.E_out = E_out; p.E_state = write_state ? c->d_E : nullptr; p.ctl = c->d_ctl;
     const int ng = (int)c->groups.size();
     p.part = c->d_epart; p.eseg = c->d_eseg; p.maxN = c->maxN;
-    p.parts = energy_parts(c->dbl, ng, std::max(c->sms, 1));
-    const int Ge = c->dbl ? std::min(c->G, 16) : c->G;
+    const int Ge = c->dbl ? std::min(c->G, 16) : c->G, sms = std::max(c->sms, 1);
+    p.tiles = energy_tiles(c->dbl, c->maxN, ng, sms);
+    p.parts = energy_parts(c->dbl, c->maxN, Ge, ng, sms);
     CK(launch_energy(c->dbl, Ge, p, ng, c->maxN, c->stream));
     return PT_OK;
 }
@@ -1435,7 +1436,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
         size_t parts = 0;  // of every grouping a shape of this context can make
         for (int g : {8, 16, 32}) {
             const int ng = S * ((chains_ps + g - 1) / g);
-            parts = std::max(parts, (size_t)ng * energy_parts(c->dbl, ng, std::max(sms, 1)));
+            parts = std::max(parts, (size_t)ng * energy_parts(c->dbl, c->maxN, g, ng, std::max(sms, 1)));
         }
         RC(dalloc(c, &c->d_epart, parts * 32));
     }

@@ -69,6 +69,7 @@ struct EnergyParams {
     Control *ctl;
     double *part;    // partial sums [group][part][32]
     int parts;       // thread blocks per group (energy_parts)
+    bool tiles;      // FP32: on energy_tile_kernel (energy_tiles)
     const int *eseg; // FP32, per sample: prefix count over the tiles (blocks) of their runs of modes (nblk+1, at seg_off)
     int maxN;
 };

@@ -40,16 +40,24 @@ PT_HD inline void replica_pair(int64_t at, int R, int *r1, int *r2) {
     *r2 = (int)(r + 1 + (at - row(r)));
 }
 
-// Thread blocks a group's full energy is split over, their partial sums added in a fixed order by a second kernel.  FP64: about
-// 8 blocks per SM (it waits on coupling loads).  FP32: one block per SM at a time, so the number of parts that leaves the least
-// of the last wave idle, each part counted with the 2% that loading the group's tables takes.
+// Whether the full energies of comb chains run on the tiles of pt_energy.cu (FP32) or on blocks of (mode, block) items.  Tiles,
+// but for small N with more groups than SMs: a tile block has an SM to itself and below N = 32 mostly waits, while 3 of the
+// other fit (GB300, the kernel alone, 65536 chains: N = 4 66 us against 30, N = 16 131 against 68; 16384 chains of N = 32 73
+// against 77; with few groups the tiles win at every N, N = 16, 160 chains 22 against 27 with its surroundings).
+inline bool energy_tiles(bool fp64, int maxN, int groups, int sms) { return !fp64 && (maxN >= 32 || groups <= sms); }
+
+// Thread blocks a group's full energy is split over, their partial sums added in a fixed order by a second kernel.  Items: about
+// 8 blocks per SM (they wait on coupling loads).  Tiles: one block per SM at a time, so the number of parts that takes the
+// least time in rounds of blocks: a block costs a + w / parts us, a for the group's tables, w for its tiles (fitted on GB300 to
+// N = 4 ... 256 and groups of 8, 16 and 32: N = 16 a 2.2 ... 3, w 1 ... 4; N = 64 3.4 ... 5.9, 20 ... 56; N = 256, groups of 8, 25, 495).
 constexpr int kEnergyPartsMax = 16;
-inline int energy_parts(bool fp64, int groups, int sms) {
-    if (fp64) return std::max(1, std::min(8, (8 * sms + groups - 1) / std::max(groups, 1)));
-    double best = 1e30;
+inline int energy_parts(bool fp64, int maxN, int G, int groups, int sms) {
+    if (!energy_tiles(fp64, maxN, groups, sms)) return std::max(1, std::min(8, (8 * sms + groups - 1) / std::max(groups, 1)));
+    const double n2 = (double)maxN * maxN, a = 2.0 + n2 * (G + 8) / 48000.0, w = 4.0e-5 * n2 * std::sqrt((double)maxN) * (G + 4);
+    double best = 1e300;
     int parts = 1;
     for (int q = 1; q <= kEnergyPartsMax; ++q) {
-        const double t = (double)(((int64_t)groups * q + sms - 1) / sms) / q * (1.0 + 0.02 * q);
+        const double t = (double)(((int64_t)groups * q + sms - 1) / sms) * (a + w / q);
         if (t < best) { best = t; parts = q; }
     }
     return parts;

@@ -733,8 +733,9 @@ __global__ void fields_kernel(FieldsParams prm) {
 // which visits every quadruplet once, at its smallest mode x (partner m: the largest; the pair {p, q} of
 // the two middle modes has p > x).  A group's share is split over prm.parts thread blocks, each writing per-chain FP64
 // sums to prm.part, and energy_sum_kernel adds the parts in order.  With renorm != 0, renorm_kernel first rescales every
-// chain onto sum |a|^4 = N.  FP32 chains: energy_tile_kernel (pt_energy.cu).  FP64: energy_kernel, whose work items are
-// (mode, block); it waits on coupling loads from L2, so it runs about 8 blocks per SM in all.
+// chain onto sum |a|^4 = N.  FP32 chains: energy_tile_kernel (pt_energy.cu), but for many groups of small N (energy_tiles).
+// Those and FP64: energy_kernel, whose work items are (mode, block); it waits on coupling loads from L2, so it runs about 8
+// blocks per SM in all.
 template <typename real, int G>
 __global__ void __launch_bounds__(256) renorm_kernel(EnergyParams prm) {
     using V = typename vec2<real>::type;
@@ -763,7 +764,7 @@ __global__ void __launch_bounds__(256) renorm_kernel(EnergyParams prm) {
 }
 
 template <typename real, int G>
-__global__ void __launch_bounds__(256, 2) energy_kernel(EnergyParams prm) {
+__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2) energy_kernel(EnergyParams prm) {
     using V = typename vec2<real>::type;
     constexpr int RS = RowStride<real, G>::value, NCW = 8, WPW = 32 / G, NW = NCW * WPW;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -939,15 +940,14 @@ template <typename real, int G>
 static cudaError_t launch_energy_t(const EnergyParams &p, int ngroups, int maxN, cudaStream_t s) {
     using V = typename vec2<real>::type;
     const size_t sm = (size_t)(maxN + 2 * APAD) * RowStride<real, G>::value * sizeof(V) + 8 * G * sizeof(double) + 64;
-    cudaError_t e = cudaSuccess;
-    if constexpr (sizeof(real) == 8) e = cudaFuncSetAttribute(energy_kernel<real, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = p.tiles ? cudaSuccess : cudaFuncSetAttribute(energy_kernel<real, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     if (p.parts < 1 || p.parts > kEnergyPartsMax || !p.part) return cudaErrorInvalidValue;
     if (p.renorm) {
         renorm_kernel<real, G><<<ngroups, 256, 0, s>>>(p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if constexpr (sizeof(real) == 4) e = launch_energy_tiles(G, p, ngroups, s);
+    if (p.tiles) e = launch_energy_tiles(G, p, ngroups, s);
     else {
         energy_kernel<real, G><<<ngroups * p.parts, 256, sm, s>>>(p);
         e = cudaGetLastError();

@@ -17,6 +17,8 @@ void replica_pair_(int64_t at, int R, int *r1, int *r2) { replica_pair(at, R, r1
 int unit_sweeps_(int seg, int sweeps, int groups) { return unit_sweeps(seg, sweeps, groups); }
 int sweep_runs_(int groups, int most, int64_t updates, int maxN) { return sweep_runs(groups, most, updates, maxN); }
 int64_t snapshot_bytes_(int n, int64_t a, int real) { return (int64_t)snapshot_bytes(n, a, (size_t)real); }
+int energy_parts_(int fp64, int maxN, int G, int groups, int sms) { return energy_parts(fp64, maxN, G, groups, sms); }
+int energy_tiles_(int fp64, int maxN, int groups, int sms) { return energy_tiles(fp64, maxN, groups, sms); }
 }
 """
 
@@ -93,3 +95,19 @@ def test_snapshots_hold_a_readout(rules, n, a, real, pieces):
     """A state of a FP64 pairs passes through the snapshot buffer in this many pieces."""
     room = rules.snapshot_bytes_(n, a, real)
     assert room >= n * a * 2 * real and -(-a // (room // 16)) == pieces
+
+
+@pytest.mark.parametrize("fp64", [0, 1])
+@pytest.mark.parametrize("N", [4, 16, 30, 32, 64, 128, 256, 512])
+@pytest.mark.parametrize("G", [8, 16, 32])
+def test_parts_of_a_full_energy(rules, fp64, N, G):
+    """Any number of groups has a valid number of parts; FP32 tiles of small N are not split where the groups fill the SMs
+    anyway (a block's tables cost more than its share of the tiles), few groups are split to fill them."""
+    for groups in (1, 3, 100, 152, 153, 160, 256, 2048, 1 << 25):
+        q = rules.energy_parts_(fp64, N, G, groups, 152)
+        assert 1 <= q <= (16 if rules.energy_tiles_(fp64, N, groups, 152) else 8)
+        if not fp64 and groups == 256 and 32 <= N <= 64:
+            assert q <= 2
+        if groups == 1:
+            assert q == (16 if not fp64 else 8)
+    assert rules.energy_tiles_(fp64, N, 152, 152) == (not fp64) and rules.energy_tiles_(fp64, N, 153, 152) == (not fp64 and N >= 32)
