@@ -147,9 +147,62 @@ __global__ void __launch_bounds__(32) swap_kernel(SwapParams p) {
     }
 }
 
+// Many ladders of at most L temperatures, L lanes each: the same steps on values that the lanes hold, exchanged by shuffles.  A
+// warp per ladder leaves nearly all lanes idle there (GB300, us per pass with a thread per ladder that takes every step alone / a
+// warp / here: 4000 ladders of 2 temperatures 15 / 19 / 14, 100000 171 / 231 / 136, 10000 of 3 29 / 35 / 24; 100 of 3 11 / 10 /
+// 13, so few ladders keep their warps; from 5 temperatures on the warp beats the thread at every count, 10000 ladders 40 / 45).
+constexpr int kSwapShort = 4, kSwapMany = 2000;
+
+template <int L> __global__ void __launch_bounds__(128) swap_short_kernel(SwapParams p) {
+    const int64_t ladder = ((int64_t)blockIdx.x * 128 + threadIdx.x) / L;
+    const int i = threadIdx.x % L, s = (int)(ladder / p.R);
+    const bool mine = ladder < (int64_t)p.S * p.R && i < p.nT;  // the others only take part in the shuffles
+    int *perm = p.perm + ladder * p.nT;
+    const int64_t pair = ladder * (p.nT - 1) + i;
+    int slot = 0;
+    double E = 0.0, b = 0.0, lu = 0.0;
+    if (mine) {
+        slot = perm[i];
+        E = p.E[slot];
+        b = p.beta[i];
+        if (i + 1 < p.nT) lu = log(u01(draw(p.seed, (uint32_t)ladder, (uint32_t)p.ctl->swap_passes, (uint32_t)i, kTagSwap).x));
+        atomicAdd(p.mcT_acc + (int64_t)s * p.nT + i, p.mc_acc[slot]);
+        atomicAdd(p.mcT_att + (int64_t)s * p.nT + i, p.mc_att[slot]);
+        p.mc_acc[slot] = 0ull;
+        p.mc_att[slot] = 0ull;
+    }
+    const unsigned all = 0xffffffffu;
+    int c0 = __shfl_sync(all, slot, 0, L), kept = slot;
+    double e0 = __shfl_sync(all, E, 0, L);
+    bool swapped = false;
+    for (int k = 0; k + 1 < p.nT; ++k) {
+        const int c1 = __shfl_sync(all, slot, k + 1, L);
+        const double e1 = __shfl_sync(all, E, k + 1, L), db = __shfl_sync(all, b, k, L) - __shfl_sync(all, b, k + 1, L);
+        const double D = db * (e0 - e1);
+        const bool swap = D >= 0.0 || __shfl_sync(all, lu, k, L) < D;
+        if (i == k) { kept = swap ? c1 : c0; swapped = swap; }
+        if (!swap) { c0 = c1; e0 = e1; }
+    }
+    if (!mine) return;
+    if (i + 1 == p.nT) kept = c0;
+    perm[i] = kept;
+    p.label[kept] = i;
+    if (i + 1 < p.nT) {
+        p.swap_att[pair] += 1ull;
+        if (swapped) p.swap_acc[pair] += 1ull;
+    }
+}
+
+template <int L> static cudaError_t launch_swap_short(const SwapParams &p, int n, cudaStream_t s) {
+    swap_short_kernel<L><<<(unsigned)(((int64_t)n * L + 127) / 128), 128, 0, s>>>(p);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_swap(const SwapParams &p, cudaStream_t s) {
     const int n = p.S * p.R;
     if (n <= 0 || p.nT < 2) return cudaSuccess;
+    if (n > kSwapMany && p.nT <= 2) return launch_swap_short<2>(p, n, s);
+    if (n > kSwapMany && p.nT <= kSwapShort) return launch_swap_short<kSwapShort>(p, n, s);
     swap_kernel<<<n, 32, 0, s>>>(p);
     return cudaGetLastError();
 }
