@@ -1,12 +1,18 @@
-"""One-chain-per-block sweeps (pt_row.cu) at the limits of their range: limits on the blocks per
+"""One-chain-per-block sweeps (pt_row.cu) at the limits of their range: the longer FP32 rows (N = 34 ... 48), limits on the blocks per
 SM, which keep an ensemble on the J-sharing blocks, the smallest N, and temperatures whose inverse is infinite."""
 import numpy as np
 import pytest
 
 import paper_2511_13508_gb300 as pkg
+import test_gpu_row
 from paper_2511_13508_gb300 import workload
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("Ns,G", [([34, 6], 8), ([48, 34, 16], 8), ([40], 16)], ids=str)
+def test_long_fp32_rows_follow_the_block_kernel(Ns, G):
+    test_gpu_row.test_row_kernel_follows_the_block_kernel("fp32", Ns, G)
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32", "fp64_plain"])

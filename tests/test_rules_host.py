@@ -111,3 +111,10 @@ def test_parts_of_a_full_energy(rules, fp64, N, G):
         if groups == 1:
             assert q == (16 if not fp64 else 8)
     assert rules.energy_tiles_(fp64, N, 152, 152) == (not fp64) and rules.energy_tiles_(fp64, N, 153, 152) == (not fp64 and N >= 32)
+
+
+@pytest.mark.parametrize("N,sweeps", [(48, 3), (64, 7), (64, 3), (128, 7)])
+def test_a_few_groups_too_many_are_cut_inside_sweeps(rules, N, sweeps):
+    """160 groups on 152 SMs, launches of test_gpu_comb_runs: runs whose ends are no ends of sweeps."""
+    runs = rules.sweep_runs_(160, 152, sweeps * N // 2, N)
+    assert runs > 1 and sweeps % runs
