@@ -135,7 +135,6 @@ struct MeasureParams {
 };
 cudaError_t launch_measure(const MeasureParams &p, cudaStream_t s);
 
-// Plain FP64 path: the paper's design restated (one block per chain, one thread per quadruplet term).
 // pt_graph.cu: FP32 sweep / energy on explicit interaction lists (one block per group of 8 chains)
 // Row stride (in float2) of the FP32 group kernels' amplitude table: the 8 chains, unpadded.  The incidence records
 // hold partner modes as row offsets (mode x this).
@@ -215,6 +214,7 @@ cudaError_t launch_row_pack(bool dbl, const SampleDev *samples, int S, const int
                             cudaStream_t s);
 cudaError_t launch_row_sweep(bool dbl, const RowParams &p, cudaStream_t s);
 
+// Plain FP64 path: the paper's design restated (one block per chain, one thread per quadruplet term).
 struct PlainParams {
     const SampleDev *samples;
     const int *chain_sample;

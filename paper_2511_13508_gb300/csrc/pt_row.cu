@@ -343,13 +343,13 @@ size_t row_smem_bytes(bool dbl, int maxN) { return dbl ? RowSmem<double>(maxN).t
 // chains FP32 8.0 (17.1); N = 32, 168 chains FP32 14.3 (32).  What is left of an update of few rows is a chain of FP64
 // latencies (about 70 clocks each); a third warp for the random numbers alone gained 5% there and cost as much at FP32.
 // Variants by the largest N: rows of at most 8 or 16 pairs keep their couplings in registers; longer rows load them in
-// eights.  The register budget follows the blocks an SM holds at that N (pair products of 227 KB).
+// eights.  The register budget follows the blocks an SM holds at that N (pair products of 227 KB).  FP32 rows end at N = 48.
 #define PT_ROW_DISPATCH(T, CALL)                                                                      \
     constexpr bool kF = sizeof(T) == 4;                                                               \
     if (maxN <= 16) { auto *k = row_sweep_kernel<T, 8, 64, kF ? 8 : 10>; CALL; }                     \
     else if (maxN <= 32) { auto *k = row_sweep_kernel<T, 16, 96, kF ? 7 : 6>; CALL; }                 \
     else if (maxN <= 64) { auto *k = row_sweep_kernel<T, 0, 160, kF ? 5 : 6>; CALL; }                 \
-    else { auto *k = row_sweep_kernel<T, 0, kRowMaxThreads, 1>; CALL; }
+    else { auto *k = row_sweep_kernel<T, 0, kF ? 160 : kRowMaxThreads, kF ? 5 : 1>; CALL; }
 
 // The limit is the kernel's largest (kRowSmemMax), not this context's: contexts of other sizes launch the same kernel.
 cudaError_t row_prepare(bool dbl, int maxN) {
