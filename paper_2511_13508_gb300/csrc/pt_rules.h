@@ -76,17 +76,23 @@ inline int unit_sweeps(int seg, int sweeps, int groups) {
 // round of units idle.  A unit costs about 8 us beside its updates (tables, amplitudes, the first couplings), an update of
 // the largest N about 2 + N^2 / 6000 us (GB300).  Measured there against one run per group and sweep (192 groups of
 // N = 256 on 152 SMs): 2298 -> 2127 us per sweep at 8 sweeps a launch, where the second round left 112 SMs idle.
+// A run is no longer than about kUnitUs, however many sweeps the launch has: in a ragged ensemble the next run of a large group
+// may be taken up while the one before still works, and that wait gives up after 10 s (kWaitNs).  Groups that all fit at once
+// keep one run, which nobody waits for.
+constexpr double kUnitUs = 1e6;
 inline int sweep_runs(int groups, int most, int64_t updates, int maxN) {
+    if (groups <= most) return 1;
     const double group_us = (double)updates * (2.0 + maxN * (double)maxN / 6000.0);
-    const int top = (int)std::max<int64_t>(1, std::min<int64_t>({updates, 512, kUnitsMax / std::max(groups, 1)}));
-    int best = 1;
+    const int64_t cap = std::max<int64_t>(1, std::min<int64_t>(updates, kUnitsMax / std::max(groups, 1)));
+    const int64_t least = std::min<int64_t>(cap, 1 + (int64_t)(group_us / kUnitUs)), top = std::min<int64_t>(cap, std::max<int64_t>(512, 2 * least));
+    int64_t best = least;
     double best_t = 1e300;
-    for (int k = 1; k <= top; ++k) {
+    for (int64_t k = least; k <= top; ++k) {
         const int64_t rounds = std::max<int64_t>(k, ((int64_t)groups * k + most - 1) / std::max(most, 1));  // runs of a group queue up
-        const double t = (double)rounds * (group_us / k + 8.0);
+        const double t = (double)rounds * (group_us / (double)k + 8.0);
         if (t < best_t) { best_t = t; best = k; }
     }
-    return best;
+    return (int)best;
 }
 
 // Bytes of the snapshot buffer: n_snap states of the chains (pairs of reals).  A host readout passes through it widened to FP64, in

@@ -118,3 +118,12 @@ def test_a_few_groups_too_many_are_cut_inside_sweeps(rules, N, sweeps):
     """160 groups on 152 SMs, launches of test_gpu_comb_runs: runs whose ends are no ends of sweeps."""
     runs = rules.sweep_runs_(160, 152, sweeps * N // 2, N)
     assert runs > 1 and sweeps % runs
+
+
+@pytest.mark.parametrize("groups,most", [(153, 152), (192, 152), (5000, 152), (40, 8)])
+@pytest.mark.parametrize("updates,N", [(1 << 30, 64), (1 << 30, 256), (100000 * 128, 256), (1 << 30, 512), (20, 4)])
+def test_a_run_is_short_beside_the_bound_on_waits(rules, groups, most, updates, N):
+    """A unit waits 10 s at most for the run before it, so a run stays near a second (an update 2 + N^2 / 6000 us)."""
+    runs = rules.sweep_runs_(groups, most, updates, N)
+    assert 1 <= runs <= updates and runs * groups <= 1 << 30
+    assert updates / runs * (2 + N * N / 6000) <= 1.01e6
