@@ -292,6 +292,10 @@ template <typename T> int dalloc(pt_ctx *c, T **out, size_t count) {
     return PT_OK;
 }
 
+// Waits for the copies of cudaMemcpy.  One from pageable memory may return while the transfer is under way, on the legacy
+// stream, for which the context's stream (a non-blocking one) does not wait: before a kernel there reads what was copied.
+cudaError_t uploads_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 template <typename T> int upload(pt_ctx *c, T *dst, const T *src, size_t count) {
     if (count == 0) return PT_OK;
     CK(cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c->stream));
@@ -764,6 +768,7 @@ int set_shape(pt_ctx *c, int G, int ncw, int spu) {
         return fail(c, PT_EUNSUPPORTED, "sweep block shape does not fit on this GPU");
     }
     CK(cudaMemcpy(c->d_groups, c->groups.data(), c->groups.size() * sizeof(GroupDev), cudaMemcpyHostToDevice));
+    CK(uploads_done());
     if (c->cfg.blocks_per_sm > 0) most = std::min(most, sms * c->cfg.blocks_per_sm);
     c->most = most;
     c->grid = std::max(1, std::min((int)c->groups.size(), most));
@@ -1419,6 +1424,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemcpy(c->d_beta, beta.data(), n_T * sizeof(double), cudaMemcpyHostToDevice));
     CK(cudaMemset(c->d_acc, 0, c->acc_words * sizeof(unsigned long long)));
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
+    CK(uploads_done());
 
     if (c->gfp32) CK(graph_prepare(graph_params(c)));
     // ---- persistent grid
@@ -1473,6 +1479,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
             std::stable_sort(order.begin(), order.end(),
                              [&](int x, int y) { return c->N[c->chain_sample[x]] > c->N[c->chain_sample[y]]; });
             CK(cudaMemcpy(c->d_order, order.data(), c->n_chains * sizeof(int), cudaMemcpyHostToDevice));
+            CK(uploads_done());
             CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
             CK(launch_row_pack(c->dbl, c->d_samples, S, quads, Jq, c->d_Jrow, c->stream));
             CK(row_prepare(c->dbl, c->maxN));
@@ -1842,6 +1849,7 @@ int pt_load(pt_ctx *c, const void *buf, size_t len) {
     ctl.swap_passes = h.swap_passes;
     ctl.global_rounds = h.global_rounds;
     CK(cudaMemcpy(c->d_ctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice));
+    CK(uploads_done());
     c->sweeps_done = h.sweeps_done;
     c->swap_passes = h.swap_passes;
     c->global_rounds = h.global_rounds;
@@ -2021,6 +2029,7 @@ int pt_learn_init(pt_ctx *c, int n_cold, int batch, int data_per_sample, uint64_
     CK(cudaMemcpy(L->M3, m3.data(), m3.size() * sizeof(float), cudaMemcpyHostToDevice));
     CK(cudaMemset(L->Am, 0, S * ps * sizeof(float)));
     CK(cudaMemset(L->Av, 0, S * ps * sizeof(float)));
+    CK(uploads_done());
     if ((rc = learn_cast(c)) != PT_OK) return rc;
     return watchdog_sync(c);
 }
@@ -2034,6 +2043,7 @@ int pt_learn_params(pt_ctx *c, float *P, int set) {
     const size_t n = (size_t)c->S * L.sh.psize;
     if (set) {
         CK(cudaMemcpy(L.P, P, n * sizeof(float), cudaMemcpyHostToDevice));
+        CK(uploads_done());
         if ((rc = learn_cast(c)) != PT_OK) return rc;
         return watchdog_sync(c);
     }
@@ -2075,6 +2085,7 @@ int pt_learn_eval(pt_ctx *c, const double *a, const int *cond, int rows, double 
     cudaError_t e = cudaMalloc(&dc, hc.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(da, a, na * sizeof(double2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dc, hc.data(), hc.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = uploads_done();
     if (e != cudaSuccess) { cudaFree(da); cudaFree(dc); return cuda_fail(c, e, "pt_learn_eval upload"); }
     FeatParams fp{};
     fp.a = da; fp.dbl = 1; fp.samples = c->d_samples; fp.slot = nullptr; fp.rows_per_sample = rows; fp.N = sh.N;
@@ -2207,6 +2218,7 @@ int pt_check_wait(pt_ctx *c, int limit_ms) {
     // clear the status the probe left, so that the context goes on
     const int zero[2] = {0, 0};
     CK(cudaMemcpy(&c->d_ctl->error, zero, sizeof(zero), cudaMemcpyHostToDevice));
+    CK(uploads_done());
     return rc;
 }
 
