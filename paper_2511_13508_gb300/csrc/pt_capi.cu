@@ -1424,7 +1424,6 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     CK(cudaMemcpy(c->d_beta, beta.data(), n_T * sizeof(double), cudaMemcpyHostToDevice));
     CK(cudaMemset(c->d_acc, 0, c->acc_words * sizeof(unsigned long long)));
     CK(cudaMemset(c->d_ctl, 0, sizeof(Control)));
-    CK(uploads_done());
 
     if (c->gfp32) CK(graph_prepare(graph_params(c)));
     // ---- persistent grid
@@ -1483,7 +1482,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
             CK(cudaMemsetAsync(c->d_Jrow, 0, (size_t)row_total * c->esize, c->stream));
             CK(launch_row_pack(c->dbl, c->d_samples, S, quads, Jq, c->d_Jrow, c->stream));
             CK(row_prepare(c->dbl, c->maxN));
-            CK(cudaStreamSynchronize(c->stream));
+            if (!keep_quads) CK(cudaStreamSynchronize(c->stream));  // the lists are given back below
         } else {
             dev_free(c, c->d_Jrow);
             dev_free(c, c->d_order);
@@ -1498,6 +1497,7 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     InitParams ip{};
     ip.samples = c->d_samples; ip.chain_sample = c->d_chain_sample; ip.label = c->d_label; ip.a = c->d_a;
     ip.dbl = c->dbl ? 1 : 0; ip.R = replicas; ip.nT = n_T; ip.seed = seed;
+    CK(uploads_done());
     CK(launch_init(ip, c->n_chains, c->stream));
     RC(run_energy(c, 0, nullptr, true));
     RC(watchdog_sync(c));
