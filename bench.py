@@ -37,11 +37,12 @@ CPU_SAMPLE_SECONDS = 15.0
 METRIC = "chain-sweeps/s at N=256 vs plain FP64; eff. samples/s learned vs plain PT"
 
 
-def flops_per_chain_sweep(N: int) -> float:
-    """Algorithmic FP32 flops of one sweep (N/2 pair updates) of the pair-factored field evaluation,
+def flops_per_chain_sweep(N: int, products: bool = True) -> float:
+    """Algorithmic flops of one sweep (N/2 pair updates) of the pair-factored field evaluation,
     averaged exactly over the pair distribution (j uniform, k uniform among the other modes):
     per pair product z = a_x a_y (6 flops) used by either field, per coupling term acc += J z (4),
-    per field row h += conj(a_m) acc (8)."""
+    per field row h += conj(a_m) acc (8).  products=False leaves the pair products out, as on the
+    one-chain-per-block kernel, which keeps them from update to update."""
     s = np.arange(2 * N - 1)
     m = np.array([max(0, (ss - 1) // 2 - max(0, ss - (N - 1)) + 1) if ss >= 1 else 0 for ss in s])
     K = np.arange(N)
@@ -55,7 +56,7 @@ def flops_per_chain_sweep(N: int) -> float:
         both = inj[None, :] & ink
         union = np.where(both, np.where(s[None, :] == j + kk[:, None], m - 1, m), np.where(inj[None, :] | ink, m - 1, 0))
         rows = (tj > 0).sum() * len(kk) + (tk > 0).sum()
-        tot += 6.0 * union.sum() + 4.0 * (tj.sum() * len(kk) + tk.sum()) + 8.0 * rows
+        tot += (6.0 * union.sum() if products else 0.0) + 4.0 * (tj.sum() * len(kk) + tk.sum()) + 8.0 * rows
     return tot / (N * (N - 1)) * (N / 2)
 
 
@@ -493,11 +494,12 @@ def workloads_leg(sweeps=64, peak32=None):
         sec = ev0.elapsed_time(ev1) / 1e3
         per_chain = W.replicas * len(W.temps)
         fl = fl_x = 0.0
+        products = prec == "fp32" or max(W.Ns) > 160  # FP64 up to N = 160 sweeps one chain per block
         for n in W.Ns:
-            if n not in fl_cache:
-                fl_cache[n] = (survey_flops_per_chain_sweep(n), flops_per_chain_sweep(n))
-            fl += fl_cache[n][0] * per_chain * sweeps
-            fl_x += fl_cache[n][1] * per_chain * sweeps
+            if (n, products) not in fl_cache:
+                fl_cache[n, products] = (survey_flops_per_chain_sweep(n), flops_per_chain_sweep(n, products))
+            fl += fl_cache[n, products][0] * per_chain * sweeps
+            fl_x += fl_cache[n, products][1] * per_chain * sweeps
         if prec == "fp32":
             peak = peak32 if peak32 else peak_fp32_tflops()
             basis = "measured FP32 FMA peak (pt_fma_probe)" if peak32 else "FP32 unit-count peak at 2070 MHz"
@@ -508,7 +510,8 @@ def workloads_leg(sweeps=64, peak32=None):
                     "chains": pt.n_chains, "N": sorted(set(int(n) for n in W.Ns)), "sweeps": sweeps,
                     "achieved_tflops": achieved, "peak_tflops": peak, "frac": achieved / peak,
                     "frac_executed": fl_x / sec / 1e12 / peak,
-                    "flop_count": "16 flops x 4|Q| per chain-sweep (frac); pair-factored executed count (frac_executed)",
+                    "flop_count": "16 flops x 4|Q| per chain-sweep (frac); pair-factored executed count, without the pair "
+                                  "products where a chain keeps them (FP64) (frac_executed)",
                     "peak_basis": basis, "autotuned_shape": list(shape) if shape else None}
         pt.close()
     return out
