@@ -134,8 +134,8 @@ def fma_probe(packed, blocks, threads, iters, sink_ptr, stream_ptr):
 
 
 def default_shape(precision, max_n, n_samples, chains_per_sample, sm_count):
-    """Sweep-block shape pt_create picks by default (pt_default_shape, host only):
-    (chains_per_block, consumer_warps)."""
+    """Sweep-block shape of a batch by size alone (pt_default_shape, host only): (chains_per_block, consumer_warps).  pt_create
+    starts from it and departs where another kernel or shape is faster: see include/pt.h."""
     G, ncw = ctypes.c_int(), ctypes.c_int()
     prec = PREC[precision] if isinstance(precision, str) else int(precision)
     _check(None, lib().pt_default_shape(prec, int(max_n), int(n_samples), int(chains_per_sample), int(sm_count),
