@@ -1270,6 +1270,8 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
     c->d_a = dev_alloc(c, (size_t)c->a_total * 2 * c->esize);
     if (!c->d_a) return bail(fail(c, PT_ENOMEM, "device allocation failed (state)"));
     c->snap_bytes = snapshot_bytes(c->n_snap_max, c->a_total, c->esize);
+    const size_t state_words = (size_t)c->a_total * 2 + c->n_chains;
+    if (state_in_one_copy(state_words)) c->snap_bytes = std::max(c->snap_bytes, state_words * sizeof(double));
     c->d_snap_a = dev_alloc(c, c->snap_bytes);
     if (!c->d_snap_a) return bail(fail(c, PT_ENOMEM, "device allocation failed (snapshots)"));
     RC(dalloc(c, &c->d_snap_E, (size_t)c->n_snap_max * c->n_chains));
@@ -1659,6 +1661,19 @@ int pt_get_state(pt_ctx *c, double *a, double *E) {
     // as that takes (one with two FP32 snapshots or an FP64 one, or up to 1 MB, else two).
     const int64_t cap = (int64_t)(c->snap_bytes / sizeof(double2));
     double2 *canon = reinterpret_cast<double2 *>(c->d_snap_a);
+    const size_t words = (size_t)c->a_total * 2 + c->n_chains;
+    if (a && E && state_in_one_copy(words)) {
+        double *out = reinterpret_cast<double *>(canon);
+        CK(launch_canon(c->d_samples, c->d_chain_sample, c->d_label, c->nT, c->d_a, c->dbl, canon, 0, c->a_total, c->d_E, out + 2 * c->a_total,
+                        c->n_chains, c->stream));
+        const int rc = watchdog_sync(c);
+        if (rc != PT_OK) return rc;
+        std::vector<double> all(words);
+        CK(cudaMemcpy(all.data(), out, words * sizeof(double), cudaMemcpyDeviceToHost));
+        std::memcpy(a, all.data(), (size_t)c->a_total * sizeof(double2));
+        std::memcpy(E, all.data() + 2 * c->a_total, c->n_chains * sizeof(double));
+        return PT_OK;
+    }
     for (int64_t lo = 0; lo == 0 || (a && lo < c->a_total); lo += cap) {
         const int64_t n = std::min(cap, c->a_total - lo);
         const bool first = lo == 0;

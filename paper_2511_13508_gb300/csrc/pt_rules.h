@@ -95,6 +95,11 @@ inline int sweep_runs(int groups, int most, int64_t updates, int maxN) {
     return (int)best;
 }
 
+// Whether amplitudes and energies (words of 8 bytes in all) come to the host in one copy and are handed out from it: while they are
+// few, a copy saved is worth more than the pass over host memory.  GB300, us a call of 4 chains, one copy / two / with the order put
+// right on the host instead of by a launch: N = 18 36 / 48 / 43, N = 64 37 / 50 / 44, N = 512 42 / 52 / 46.
+inline bool state_in_one_copy(size_t words) { return words <= 8192; }
+
 // Bytes of the snapshot buffer: n_snap states of the chains (pairs of reals).  A host readout passes through it widened to FP64, in
 // as many pieces as that takes; FP32 with one snapshot would need two, which costs a small state more than the copy itself
 // (N = 64, 12 chains: 72 us against 46 in one piece; N = 256, 96 chains: 98 against 65, on GB300), so up to 1 MB it has the room.
