@@ -1012,21 +1012,21 @@ static int create_impl(pt_ctx **out, const pt_config *cfg_in, int S, const int32
                        uint64_t seed, pt_alloc_fn alloc, pt_free_fn free_, void *alloc_user, void *stream);
 
 // Default shape of the sweep blocks (chains sharing one J stream G, field warps ncw) for the largest N, the sample
-// count and chains per sample, and the device's SM count; G_in > 0 keeps that G.  Measured on GB300
-// (chain-sweeps/s):
-// - N >= 160: 8 chains x 11 warps (N = 192, 32 samples x 64 chains: 1.48M against 1.41M with 16 x 11; N = 256,
-//   16 x 96 chains: 0.694M against 0.481M);
-// - 48 <= N < 160: the most chains per block that still give about one group per SM, from 32, 16, 8 below
-//   N = 96 and from 16, 8 above (N = 64, 64 samples x 64 chains: 32 x 11 24.2M against 20.8M with 16 x 11
-//   and 12.5M with 8 x 11; 16 samples x 64 chains: 8 x 11 10.0M against 5.7M with 32 x 11, which leaves most
-//   SMs idle; N = 128, 64 samples x 64 chains: 16 x 11 4.71M against 4.50M with 32 x 11 and 3.81M with
-//   8 x 11; the ragged batch N in {32..128}: 16 x 11 8.91M against 8.38M with 8 x 11), 32 x 11 (16 x 11 from
-//   N = 96) when none does;
+// count and chains per sample, and the device's SM count; G_in > 0 keeps that G.  Measured on GB300 (chain-sweeps/s,
+// launches of 64 sweeps, samples x chains):
+// - N >= 160: 8 chains x 11 warps (N = 192, 32 x 64: 1.54M against 1.46M with 16 x 11; N = 256, 16 x 96: 0.731M against
+//   0.499M).  At N = 160 itself many samples would gain from 16 x 11 (64 x 64: 2.78M against 2.39M);
+// - 48 <= N < 160: the most chains per block that still give about one group per SM, from 32, 16, 8 below N = 96 and from
+//   16, 8 above, 32 x 11 (16 x 11 from N = 96) when none does.  32 / 16 / 8 chains: N = 48, 64 x 64 48.1M / 39.4M / 22.5M,
+//   16 x 64 12.0M / 16.8M / 19.0M; N = 64, 64 x 64 25.9M / 22.5M / 15.5M, 32 x 64 13.0M / 19.1M / 15.4M, 16 x 64 6.5M / 9.6M /
+//   13.1M; N = 96, 64 x 64 9.90M / 9.74M / 7.19M, 32 x 64 4.95M / 8.26M / 7.17M; N = 128, 64 x 64 4.71M / 4.90M / 4.00M, 32 x 64
+//   2.36M / 4.14M / 3.99M; the ragged batch N in {32..128} 5.27M / 9.33M / 9.29M.  Launches of single sweeps go the same way but
+//   for N = 96 and 128, 64 x 64, where 32 chains gain 12 and 3%;
 // - N < 48: 16 x 7;
 // - at most 8 chains per sample: 8 chains per block.
-// Field warps: 11 from N = 48 on (N = 64, 64 samples: 32 x 11 22.3M chain-sweeps/s against 21.6M with 32 x 7;
-// ragged batch: 16 x 11 8.24M against 7.53M with 16 x 7), else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3
-// (N = 64, 64 samples: 16 x 3 685k, 8 x 7 521k).
+// Field warps: 11 from N = 48 on (N = 64, 64 x 64: 32 x 11 25.9M against 24.0M with 32 x 7; ragged batch: 16 x 11 9.33M, 16 x 7
+// 8.52M, 16 x 15 9.25M; N = 256: 8 x 11 0.731M, 8 x 7 0.646M), else 7.  FP64: 8 x 7 from N = 128 on, else 16 x 3 (N = 64, 64 x 64:
+// 16 x 3 665k, 8 x 7 469k; N = 128, 8 x 64: 20.8k, 49.5k).
 static void default_shape(bool dbl, int maxN, int S, int chains_ps, int sms, int G_in, int *G_out, int *ncw_out) {
     int G = G_in;
     if (G == 0) {

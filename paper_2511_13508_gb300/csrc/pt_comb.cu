@@ -15,7 +15,7 @@
 // Measured on GB300, us per sweep, against eight sums reduced per chain behind two barriers and one block per group with
 // whole sweeps as work units: N = 256, 16 samples of 96 chains, 8 sweeps a launch 2300 -> 2127 (the finer units); one such
 // sample 1680 -> 428 (clusters of 8); N = 64, 64 samples of 64 chains 163 -> 161; ragged N = 32 ... 128, 96 samples of 48
-// chains 510 -> 495.
+// chains 510 -> 494 in launches of 64 sweeps (505 of 8, 516 of one).
 #include <cstdint>
 #include "pt_bulk.cuh"
 #include "pt_common.cuh"

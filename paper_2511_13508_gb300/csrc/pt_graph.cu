@@ -870,7 +870,8 @@ namespace {
 // block / other kernel.  Table: sparse N = 48, 1024 and 4096 chains, 120 records 27 / 40 and 75 / 143, 186 39 / 42 and
 // 112 / 150, 268 50 / 42 and 144 / 151, 352 67 / 43 and 192 / 157.  Table of 4 chains, N = 96: 190 76 / 129 and 217 / 439,
 // 314 113 / 138 and 331 / 470.  Group kernel, N = 256: 80 91 / 292 and 275 / 1143, 272 241 / 314 and 724 / 1237, 418
-// 380 / 347 and 1145 / 1364.
+// 380 / 347 and 1145 / 1364.  Against the 8-chain table the line would lie near 200 records at 1024 chains and near 290 at 4096;
+// 256 for both gives up to 20% at one and 5% at the other.
 constexpr int kWarpMaxRec = 256, kWarpMaxAlone = 352;
 constexpr size_t kGraphSmemMax = 227 * 1024 - 8 * 1024;  // dynamic part (the static reduction table aside)
 
